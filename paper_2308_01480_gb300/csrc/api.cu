@@ -975,12 +975,14 @@ static tt_status pass_layout(int op, int64_t m, int64_t n, int b, int c_dtype, P
         xt = std::max(ttr::tc_ga_scratch_bytes(m, b), ttr::tc_proj_scratch_bytes(m, b, 0));
       } else {
         L->fused = ttr::simt_ga_fused_ok(m, b);
-        part = L->fused ? ttr::simt_ga_partials(m, n, b) : ttr::simt_cs_partials(m, n, b);
+        part = L->fused ? ttr::simt_ga_partials(m, n, b)
+                        : std::max(ttr::simt_cs_partials(m, n, b), ttr::simt_proj_splits(m, n) * b * n);
         if (!L->fused) sbuf = (size_t)b * n;
       }
       break;
     case TT_PASS_PROJECT:
       if (tc) xt = ttr::tc_proj_scratch_bytes(m, b, b <= 32 ? 1 : 0);
+      else if (ttr::simt_proj_splits(m, n) > 1) part = ttr::simt_proj_splits(m, n) * b * n;
       break;
     case TT_PASS_GRAM:
       if (m > 2048) return fail(TT_EUNSUPPORTED, "Gram pass needs m <= 2048");
@@ -1049,10 +1051,10 @@ tt_status tt_pass(int op, const void* C, int c_dtype, int64_t m, int64_t n, int 
         else TTR_CUDA(ttr::simt_ga<float>((const float*)C, m, n, x, b, b, part, (float*)y, b, st));
       } else {
         if (bf) {
-          TTR_CUDA((ttr::simt_proj<__nv_bfloat16, float>(Cb, m, n, x, b, b, sbuf, n, st)));
+          TTR_CUDA((ttr::simt_proj<__nv_bfloat16, float>(Cb, m, n, x, b, b, sbuf, n, st, part)));
           TTR_CUDA(ttr::simt_cs<__nv_bfloat16>(Cb, m, n, sbuf, n, b, part, (float*)y, b, st));
         } else {
-          TTR_CUDA((ttr::simt_proj<float, float>((const float*)C, m, n, x, b, b, sbuf, n, st)));
+          TTR_CUDA((ttr::simt_proj<float, float>((const float*)C, m, n, x, b, b, sbuf, n, st, part)));
           TTR_CUDA(ttr::simt_cs<float>((const float*)C, m, n, sbuf, n, b, part, (float*)y, b, st));
         }
       }
@@ -1061,11 +1063,11 @@ tt_status tt_pass(int op, const void* C, int c_dtype, int64_t m, int64_t n, int 
       if (L.tc) {
         TTR_CUDA(ttr::tc_proj(Cb, m, n, x, b, b, b <= 32 ? 1 : 0, y, y_dtype == TT_BF16 ? 1 : 0, n, xt, status, st));
       } else if (y_dtype == TT_BF16) {
-        if (bf) TTR_CUDA((ttr::simt_proj<__nv_bfloat16, __nv_bfloat16>(Cb, m, n, x, b, b, (__nv_bfloat16*)y, n, st)));
-        else TTR_CUDA((ttr::simt_proj<float, __nv_bfloat16>((const float*)C, m, n, x, b, b, (__nv_bfloat16*)y, n, st)));
+        if (bf) TTR_CUDA((ttr::simt_proj<__nv_bfloat16, __nv_bfloat16>(Cb, m, n, x, b, b, (__nv_bfloat16*)y, n, st, part)));
+        else TTR_CUDA((ttr::simt_proj<float, __nv_bfloat16>((const float*)C, m, n, x, b, b, (__nv_bfloat16*)y, n, st, part)));
       } else {
-        if (bf) TTR_CUDA((ttr::simt_proj<__nv_bfloat16, float>(Cb, m, n, x, b, b, (float*)y, n, st)));
-        else TTR_CUDA((ttr::simt_proj<float, float>((const float*)C, m, n, x, b, b, (float*)y, n, st)));
+        if (bf) TTR_CUDA((ttr::simt_proj<__nv_bfloat16, float>(Cb, m, n, x, b, b, (float*)y, n, st, part)));
+        else TTR_CUDA((ttr::simt_proj<float, float>((const float*)C, m, n, x, b, b, (float*)y, n, st, part)));
       }
       break;
     case TT_PASS_GRAM:

@@ -15,9 +15,8 @@
 // A second kernel sums each tile's split partials in a fixed order and
 // writes both triangles of G (deterministic, bit-reproducible).
 //
-// SIMT Gram (FP32 C, or BF16 shapes the tensor-core path does not take):
-// 64 x 64 upper-triangular tiles with 4 x 4 register tiles, split-K, the same
-// fixed-order reduction.
+// FP32 C, and BF16 shapes the tensor-core path does not take: the CUDA-core
+// tiles of stream_simt.cu.
 //
 // Power: W (m x c) = G X, FP32, X a 16-byte-aligned padded block; 8 rows of
 // W per CTA over many CTAs, four 128-row K chunks in flight by 16-byte
@@ -332,81 +331,6 @@ cudaError_t map_rows128(CUtensorMap* map, const void* base, int64_t rows, int64_
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// ------------------------------------------------------------ SIMT Gram
-constexpr int GS_T = 64;     // tile edge
-constexpr int GS_K = 32;     // columns of C per smem chunk
-
-// P[item] (64 x 64) = rows I of C times rows J of C, transposed, over the
-// item's column range; tiles I <= J enumerated J-major.
-template <typename TIn>
-__global__ void __launch_bounds__(256) k_gram_simt_tiles(const TIn* __restrict__ C, int64_t m, int64_t n,
-                                                         int splits, float* __restrict__ P) {
-  __shared__ __align__(16) float As[GS_K][GS_T + 4];
-  __shared__ __align__(16) float Bs[GS_K][GS_T + 4];
-  const int item = blockIdx.x;
-  const int t = item / splits, s = item % splits;
-  int J = 0;
-  while ((J + 1) * (J + 2) / 2 <= t) ++J;
-  const int I = t - J * (J + 1) / 2;
-  const int64_t chunks = ceil_div(n, GS_K);
-  const int64_t c0 = chunks * s / splits * GS_K, c1 = imin(n, chunks * (s + 1) / splits * GS_K);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int64_t ra = (int64_t)I * GS_T, rb = (int64_t)J * GS_T;
-  float acc[4][4] = {};
-  for (int64_t k0 = c0; k0 < c1; k0 += GS_K) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < GS_T * GS_K; e += 256) {
-      const int r = e / GS_K, kk = e % GS_K;
-      const int64_t col = k0 + kk;
-      As[kk][r] = (ra + r < m && col < c1) ? ld_elem(C, (ra + r) * n + col) : 0.f;
-      Bs[kk][r] = (rb + r < m && col < c1) ? ld_elem(C, (rb + r) * n + col) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < GS_K; ++kk) {
-      const float4 a4 = *reinterpret_cast<const float4*>(&As[kk][4 * ty]);
-      const float4 b4 = *reinterpret_cast<const float4*>(&Bs[kk][4 * tx]);
-      const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int w = 0; w < 4; ++w) acc[u][w] = fmaf(av[u], bv[w], acc[u][w]);
-    }
-  }
-  float* out = P + (size_t)item * GS_T * GS_T;
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-    *reinterpret_cast<float4*>(out + (4 * ty + u) * GS_T + 4 * tx) =
-        make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
-}
-
-__global__ void k_gram_simt_reduce(const float* __restrict__ P, int64_t m, int splits, float* __restrict__ G) {
-  const int i = blockIdx.y;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < i || j >= m) return;
-  const int I = i / GS_T, J = j / GS_T;
-  const int t = J * (J + 1) / 2 + I;
-  const float* src = P + (size_t)t * splits * GS_T * GS_T + (size_t)(i - GS_T * I) * GS_T + (j - GS_T * J);
-  float s0 = 0.f, s1 = 0.f;
-  int k = 0;
-  for (; k + 2 <= splits; k += 2) {
-    s0 += src[(size_t)k * GS_T * GS_T];
-    s1 += src[(size_t)(k + 1) * GS_T * GS_T];
-  }
-  if (k < splits) s0 += src[(size_t)k * GS_T * GS_T];
-  const float s = s0 + s1;
-  G[(int64_t)i * m + j] = s;
-  if (j != i) G[(int64_t)j * m + i] = s;
-}
-
-void gs_plan(int64_t m, int64_t n, int* tiles, int* splits) {
-  const int nT = (int)ceil_div(m, GS_T);
-  *tiles = nT * (nT + 1) / 2;
-  const int64_t chunks = ceil_div(n, GS_K);
-  const int want = (int)ceil_div(4 * (int64_t)num_sms_gram(), *tiles);
-  *splits = (int)imax(1, imin(imin(want, chunks), 64));
-}
-
 // ------------------------------------------------------------ power W = G X
 // X is a padded block (m x ldx, ldx % 4 == 0, 16-byte aligned), so both
 // operands arrive by 16-byte asynchronous copies, GP_ST chunks of 128 rows of
@@ -533,9 +457,7 @@ size_t gram_tiled_partials(int64_t m, int64_t n, int c_bf16) {
     if (!gt_plan(m, n, p)) return 0;
     return (size_t)p.nitems * 128 * 256;
   }
-  int tiles, splits;
-  gs_plan(m, n, &tiles, &splits);
-  return (size_t)tiles * splits * GS_T * GS_T;
+  return (size_t)simt_gram_partials(m, n);
 }
 
 cudaError_t gram_tiled(const void* C, int c_bf16, int64_t m, int64_t n, float* partials, float* G, int* status,
@@ -564,22 +486,8 @@ cudaError_t gram_tiled(const void* C, int c_bf16, int64_t m, int64_t n, float* p
     k_gram_tiles_reduce<<<dim3((unsigned)ceil_div(m, 256), (unsigned)m), 256, 0, st>>>(p, G);
     return cudaGetLastError();
   }
-  int tiles, splits;
-  gs_plan(m, n, &tiles, &splits);
-  {
-    ProfScope prof("gram_simt_tiled", st, bytes, flops);
-    note_launch("gram_simt_tiled");
-    if (c_bf16)
-      k_gram_simt_tiles<__nv_bfloat16><<<tiles * splits, 256, 0, st>>>((const __nv_bfloat16*)C, m, n, splits,
-                                                                        partials);
-    else
-      k_gram_simt_tiles<float><<<tiles * splits, 256, 0, st>>>((const float*)C, m, n, splits, partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  note_launch("gram_reduce");
-  k_gram_simt_reduce<<<dim3((unsigned)ceil_div(m, 256), (unsigned)m), 256, 0, st>>>(partials, m, splits, G);
-  return cudaGetLastError();
+  if (c_bf16) return simt_gram((const __nv_bfloat16*)C, m, n, partials, G, st, "gram_simt_tiled");
+  return simt_gram((const float*)C, m, n, partials, G, st, "gram_simt_tiled");
 }
 
 bool gram_power_ok(int64_t m, int c) { return m >= 1 && c >= 1 && c <= 64; }

@@ -30,9 +30,9 @@ class ProfScope {
   bool timed_ = false;
 };
 
-// ---- SIMT streaming passes (stream_simt.cu)
+// ---- SIMT streaming passes (stream_simt.cu, stream_proj.cu, stream_ga.cuh)
 // partials (optional): b x n x simt_proj_splits(m, n) floats enabling the
-// row-split form for tall-thin unfoldings
+// form that splits the rows over the grid
 template <typename TIn, typename TOut>
 cudaError_t simt_proj(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b, TOut* S,
                       int64_t lds, cudaStream_t st, float* partials = nullptr);
@@ -44,7 +44,8 @@ template <typename TIn>
 cudaError_t simt_ga(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b,
                     float* partials, float* out, int64_t ldo, cudaStream_t st);
 template <typename TIn>
-cudaError_t simt_gram(const TIn* C, int64_t m, int64_t n, float* partials, float* out, cudaStream_t st);
+cudaError_t simt_gram(const TIn* C, int64_t m, int64_t n, float* partials, float* out, cudaStream_t st,
+                      const char* family = "gram_simt");
 template <typename TIn>
 cudaError_t simt_ga_with_ctas(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b,
                               float* partials, int64_t max_ctas, float* out, int64_t ldo, cudaStream_t st);

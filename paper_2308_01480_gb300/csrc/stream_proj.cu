@@ -1,0 +1,262 @@
+// CUDA-core projection S = X^T C (Alg. 3 step 10, and the first half of a
+// Krylov power for tall unfoldings): the FP32 form, and BF16 unfoldings the
+// tensor-core pass does not take.
+//
+// Every column of C is one column of S, so a thread keeps four whole
+// columns (TC sums of each) in registers and reads C straight from global
+// memory, coalesced along the row: C needs no shared memory and no barrier.  X is the small operand: chunks of 64 rows are double-buffered in
+// shared memory and read as broadcasts, one 16-byte load for 16
+// multiply-adds.  The next rows of C (16 to 32 elements a thread) are in
+// flight while the current ones are multiplied.
+// The eight warps of a CTA split into CG groups of output rows (b > 20), RG
+// groups of rows of C (few columns: the groups' sums are added in order) and
+// the rest over columns; when even that leaves the chip idle (n below
+// 128 x 152 columns), the rows are also split over the grid and a second
+// kernel adds the partials in split order.
+// Measured (FP32, us; before: 16 x 16 threads with both operands staged in
+// shared memory and no split over rows unless n <= 512): 7680 x 2048 at
+// b = 20 440 -> 31, 800 x 64,000 at b = 20 ~120 -> 106, 45 x 4,100,625 at
+// b = 4 ~600 -> 170.  What bounds it now is the issue rate (53 of every 100
+// instructions are multiply-adds, one CTA an SM at b = 20).
+#include "cluster_la.cuh"
+#include "common.cuh"
+#include "kernels.h"
+
+namespace ttr {
+
+namespace {
+
+constexpr int PJ_RK = 64;   // rows of X per shared-memory chunk
+constexpr int PJ_NC = 4;    // columns of C per thread
+
+__device__ __forceinline__ void cp_async16z(float* dst, const float* src, bool ok) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+
+// vec: every row of C (and of S) starts aligned to four elements, and the
+// thread's columns are neighbours; otherwise they are 32 apart.  x16: rows
+// of X are 16-byte aligned and b is a multiple of four.
+template <typename TIn, typename TOut, int TC, int FR, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) k_proj(const TIn* __restrict__ C, int64_t m, int64_t n,
+                                                    const float* __restrict__ X, int ldx, int b,
+                                                    TOut* __restrict__ S, int64_t lds, int64_t rows_per,
+                                                    int64_t split_stride, int CG, int RG, bool vec, bool x16) {
+  constexpr int NC = PJ_NC;
+  extern __shared__ __align__(16) float pj_sm[];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int CW = 8 / (CG * RG);
+  const int cw = w % CW, cg = (w / CW) % CG, rg = w / (CW * CG);
+  const int BP = CG * TC;
+  const int64_t col = (int64_t)blockIdx.x * (CW * 32 * NC) + cw * (32 * NC) + (vec ? NC * lane : lane);
+  const int64_t rbeg = (int64_t)blockIdx.y * rows_per, rend = imin(m, rbeg + rows_per);
+  S += (int64_t)blockIdx.y * split_stride;
+  const int per_group = PJ_RK / RG;             // rows of a chunk that one group takes
+  const int nchunk = (int)ceil_div(rend - rbeg, PJ_RK);
+  bool in[NC];
+#pragma unroll
+  for (int u = 0; u < NC; ++u) in[u] = vec ? col < n : col + 32 * u < n;   // vec: all four or none
+  auto stage = [&](int ch) {
+    float* xs = pj_sm + (ch & 1) * PJ_RK * BP;
+    const int64_t i0 = rbeg + (int64_t)ch * PJ_RK;
+    if (x16) {
+      const int q = BP / 4;
+      for (int e = tid; e < PJ_RK * q; e += 256) {
+        const int r = e / q, c = (e - r * q) * 4;
+        const bool ok = i0 + r < rend && c < b;
+        cp_async16z(xs + 4 * e, ok ? X + (i0 + r) * ldx + c : X, ok);
+      }
+    } else {
+      for (int e = tid; e < PJ_RK * BP; e += 256) {
+        const int r = e / BP, c = e - r * BP;
+        const bool ok = i0 + r < rend && c < b;
+        cp_async4(xs + e, ok ? X + (i0 + r) * ldx + c : X, ok);
+      }
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  auto fetch = [&](float (&v)[FR][NC], int64_t i0) {
+    const TIn* p = C + i0 * n + col;
+    const int left = (int)imin(FR, rend - i0);
+#pragma unroll
+    for (int r = 0; r < FR; ++r) {
+      if (vec) {
+#pragma unroll
+        for (int u = 0; u < NC; ++u) v[r][u] = 0.f;
+        if (r < left && in[0]) ld4(p, v[r]);
+      } else {
+#pragma unroll
+        for (int u = 0; u < NC; ++u) v[r][u] = (r < left && in[u]) ? ld_elem(p, 32 * u) : 0.f;
+      }
+      p += n;
+    }
+  };
+  float acc[NC][TC];
+#pragma unroll
+  for (int u = 0; u < NC; ++u)
+#pragma unroll
+    for (int c = 0; c < TC; ++c) acc[u][c] = 0.f;
+  float cur[FR][NC], nxt[FR][NC] = {};
+  stage(0);
+  const int64_t g0 = rbeg + rg * per_group;     // the group's first row
+  fetch(cur, g0);
+  for (int ch = 0; ch < nchunk; ++ch) {
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();
+    if (ch + 1 < nchunk) stage(ch + 1);
+    const int64_t i0 = g0 + (int64_t)ch * PJ_RK;
+    const int rows = (int)imin(per_group, rend - i0);
+    const float* xs = pj_sm + (ch & 1) * PJ_RK * BP + (size_t)rg * per_group * BP + cg * TC;
+    for (int s = 0; s < rows; s += FR) {
+      const bool more = s + FR < rows;
+      if (more || ch + 1 < nchunk) fetch(nxt, more ? i0 + s + FR : i0 + PJ_RK);
+#pragma unroll
+      for (int r = 0; r < FR; ++r)
+#pragma unroll
+        for (int c4 = 0; c4 < TC / 4; ++c4) {
+          const float4 x = *reinterpret_cast<const float4*>(xs + (s + r) * BP + 4 * c4);
+#pragma unroll
+          for (int u = 0; u < NC; ++u) {
+            acc[u][4 * c4] = fmaf(x.x, cur[r][u], acc[u][4 * c4]);
+            acc[u][4 * c4 + 1] = fmaf(x.y, cur[r][u], acc[u][4 * c4 + 1]);
+            acc[u][4 * c4 + 2] = fmaf(x.z, cur[r][u], acc[u][4 * c4 + 2]);
+            acc[u][4 * c4 + 3] = fmaf(x.w, cur[r][u], acc[u][4 * c4 + 3]);
+          }
+        }
+#pragma unroll
+      for (int r = 0; r < FR; ++r)
+#pragma unroll
+        for (int u = 0; u < NC; ++u) cur[r][u] = nxt[r][u];
+    }
+  }
+  // sums of the row groups, added in group order
+  const int gt = 256 / RG;                      // threads of one group
+  const int t = tid % gt;
+  for (int g = 1; g < RG; ++g) {
+    __syncthreads();
+    if (rg == g) {
+#pragma unroll
+      for (int u = 0; u < NC; ++u)
+#pragma unroll
+        for (int c = 0; c < TC; ++c) pj_sm[(u * TC + c) * gt + t] = acc[u][c];
+    }
+    __syncthreads();
+    if (rg == 0) {
+#pragma unroll
+      for (int u = 0; u < NC; ++u)
+#pragma unroll
+        for (int c = 0; c < TC; ++c) acc[u][c] += pj_sm[(u * TC + c) * gt + t];
+    }
+  }
+  if (rg != 0) return;
+#pragma unroll
+  for (int c = 0; c < TC; ++c) {
+    const int row = cg * TC + c;
+    if (row < b) {
+      TOut* out = S + (int64_t)row * lds + col;
+      if (vec) {
+        const float v[4] = {acc[0][c], acc[1][c], acc[2][c], acc[3][c]};
+        if (in[0]) st4(out, v);
+      } else {
+#pragma unroll
+        for (int u = 0; u < NC; ++u)
+          if (in[u]) st_elem(out, 32 * u, acc[u][c]);
+      }
+    }
+  }
+}
+
+// S (b x n) = sum over row splits of the partials P[y] (b x n), fixed order.
+template <typename TOut>
+__global__ void k_sum_splits(const float* __restrict__ P, int splits, int b, int64_t n, TOut* __restrict__ S,
+                             int64_t lds) {
+  const int64_t E = (int64_t)b * n;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x) {
+    // eight loads in flight, added in split order
+    float acc = 0.f;
+    int y = 0;
+    for (; y + 8 <= splits; y += 8) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = P[(int64_t)(y + u) * E + e];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc += v[u];
+    }
+    for (; y < splits; ++y) acc += P[(int64_t)y * E + e];
+    st_elem(S, (e / n) * lds + e % n, acc);
+  }
+}
+
+template <typename TIn, typename TOut, int TC>
+cudaError_t launch_proj(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b, TOut* S, int64_t lds,
+                        int64_t rows_per, int splits, int64_t split_stride, int CG, cudaStream_t st) {
+  constexpr int NC = PJ_NC;
+  // narrow outputs: more CTAs an SM; the widest holds its 80 sums and 64
+  // loads in one
+  constexpr int FR = TC >= 20 ? 8 : 4, CTAS = TC >= 20 ? 1 : TC >= 12 ? 2 : 3;
+  // as few row groups as give the chip two CTAs an SM
+  int RG = 1;
+  while (CG * RG < 8 && rows_per >= 16 * RG && ceil_div(n, (8 / (CG * RG)) * 32 * NC) * splits < 2 * 152) RG *= 2;
+  const int cols = (8 / (CG * RG)) * 32 * NC;
+  const bool vec = n % 4 == 0 && lds % 4 == 0 && split_stride % 4 == 0 &&
+                   reinterpret_cast<uintptr_t>(C) % (4 * sizeof(TIn)) == 0 &&
+                   reinterpret_cast<uintptr_t>(S) % (4 * sizeof(TOut)) == 0;
+  const bool x16 = b % 4 == 0 && ldx % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0;
+  const size_t smem = sizeof(float) * (size_t)imax(2 * PJ_RK * CG * TC, RG > 1 ? (256 / RG) * NC * TC : 0);
+  k_proj<TIn, TOut, TC, FR, CTAS><<<dim3((unsigned)ceil_div(n, cols), (unsigned)splits), 256, smem, st>>>(
+      C, m, n, X, ldx, b, S, lds, rows_per, split_stride, CG, RG, vec, x16);
+  return cudaGetLastError();
+}
+
+template <typename TIn, typename TOut>
+cudaError_t proj_dispatch(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b, TOut* S, int64_t lds,
+                          int64_t rows_per, int splits, int64_t split_stride, cudaStream_t st) {
+#define TTR_PJ(TC, CG) return launch_proj<TIn, TOut, TC>(C, m, n, X, ldx, b, S, lds, rows_per, splits, split_stride, CG, st)
+  if (b <= 4) TTR_PJ(4, 1);
+  if (b <= 8) TTR_PJ(8, 1);
+  if (b <= 12) TTR_PJ(12, 1);
+  if (b <= 16) TTR_PJ(16, 1);
+  if (b <= 20) TTR_PJ(20, 1);
+  if (b <= 24) TTR_PJ(12, 2);
+  if (b <= 32) TTR_PJ(16, 2);
+  if (b <= 40) TTR_PJ(20, 2);
+  if (b <= 48) TTR_PJ(12, 4);
+  if (b <= 64) TTR_PJ(16, 4);
+#undef TTR_PJ
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+// Row splits over the grid: one when the columns alone fill the chip.
+int64_t simt_proj_splits(int64_t m, int64_t n) {
+  const int64_t wide = ceil_div(n, 128);
+  if (m < 256 || wide >= 152) return 1;
+  return imax(1, imin(imin(2 * 152 / wide, ceil_div(m, 32)), 64));
+}
+
+template <typename TIn, typename TOut>
+cudaError_t simt_proj(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b, TOut* S,
+                      int64_t lds, cudaStream_t st, float* partials) {
+  const int64_t splits0 = partials ? simt_proj_splits(m, n) : 1;
+  const int64_t rows_per = ceil_div(m, splits0), splits = ceil_div(m, rows_per);
+  ProfScope prof("proj_simt", st, (double)m * n * sizeof(TIn) + (double)m * b * 4 + (double)b * n * sizeof(TOut),
+                 2.0 * m * n * b);
+  if (splits == 1) {
+    note_launch("proj_simt");
+    return proj_dispatch<TIn, TOut>(C, m, n, X, ldx, b, S, lds, m, 1, 0, st);
+  }
+  const int64_t E = (int64_t)b * n;
+  note_launch("proj_simt", 2);
+  const cudaError_t e = proj_dispatch<TIn, float>(C, m, n, X, ldx, b, partials, n, rows_per, (int)splits, E, st);
+  if (e != cudaSuccess) return e;
+  k_sum_splits<TOut><<<(int)imin(ceil_div(E, 256), 4 * 152), 256, 0, st>>>(partials, (int)splits, b, n, S, lds);
+  return cudaGetLastError();
+}
+
+template cudaError_t simt_proj<float, float>(const float*, int64_t, int64_t, const float*, int, int, float*, int64_t, cudaStream_t, float*);
+template cudaError_t simt_proj<float, __nv_bfloat16>(const float*, int64_t, int64_t, const float*, int, int, __nv_bfloat16*, int64_t, cudaStream_t, float*);
+template cudaError_t simt_proj<__nv_bfloat16, float>(const __nv_bfloat16*, int64_t, int64_t, const float*, int, int, float*, int64_t, cudaStream_t, float*);
+template cudaError_t simt_proj<__nv_bfloat16, __nv_bfloat16>(const __nv_bfloat16*, int64_t, int64_t, const float*, int, int, __nv_bfloat16*, int64_t, cudaStream_t, float*);
+
+}  // namespace ttr

@@ -1,288 +1,99 @@
-// CUDA-core (SIMT) streaming passes over an unfolding C (m x n, row-major).
-//
-// These are the plain FP32 form of the four passes of Alg. 3 (and the form
-// used for shapes the tensor-core kernels do not cover):
-//   proj  : S = X^T C              (Alg. 3 step 10, and the first half of a
-//                                   Krylov power for tall unfoldings)
-//   cs    : Y = C S^T              (Alg. 3 step 4: the sketch C W with
-//                                   S = W^T, or the second half of a power)
-//   ga    : Y = C (C^T X)          (Alg. 3 step 4: one Krylov power, fused so
-//                                   each column tile of C is read once)
-//   gram  : G = C C^T              (exhaustion route: all of R^m is Krylov)
-// Reductions over n are split across CTAs into per-CTA partials that a
-// second kernel sums in a fixed order, so results are bit-reproducible.
+// CUDA-core (SIMT) streaming passes over an unfolding C (m x n, row-major):
+// the plain FP32 form of the passes of Alg. 3, and the form used for BF16
+// shapes the tensor-core kernels do not cover.
+//   cs    : Y = C S^T          (Alg. 3 step 4: the sketch C W with S = W^T,
+//                               or the second half of a power)
+//   gram  : G = C C^T          (exhaustion route: all of R^m is Krylov; and
+//                               the tiles of the Gram-power route)
+// (the projection is stream_proj.cu, the fused power stream_ga.cuh).
+// Both are products of rows with rows (simt_tile.cuh).  Reductions over n are
+// split across CTAs into per-CTA partials that a second kernel sums in a
+// fixed order, so results are bit-reproducible.
+// Measured (FP32, us; before: 2 x VB register tiles on scalar shared loads):
+// the sketch of 45 x 4,100,625 at b = 6 ~900 -> 184 (4.0 TB/s), of
+// 800 x 64,000 at b = 20 ~120 -> 68, of 7680 x 2048 at b = 20 91 -> 26; the
+// Gram of 32 x 1,048,576 180 -> 62, of a BF16 61 x 112,095 145 -> 48.
 #include "common.cuh"
 #include "kernels.h"
+#include "simt_tile.cuh"
 
 namespace ttr {
 
-// ---------------------------------------------------------------- proj
-// S[c][col] = sum_i X[i][c] C[i][col];  256 threads = 16 (cols) x 16 (c).
-// With gridDim.y > 1 each CTA row covers rows [y * rows_per, ...) and writes
-// its partial sums to S + y * split_stride (the tall-thin form).
-template <typename TIn, typename TOut, int VB>
-__global__ void __launch_bounds__(256) k_proj(const TIn* __restrict__ C, int64_t m, int64_t n,
-                                              const float* __restrict__ X, int ldx, int b,
-                                              TOut* __restrict__ S, int64_t lds, int64_t rows_per,
-                                              int64_t split_stride) {
-  constexpr int TN = 64, RC = 32;
-  __shared__ float Cs[RC][TN];
-  __shared__ float Xs[RC][16 * VB];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int64_t col0 = (int64_t)blockIdx.x * TN;
-  const int64_t rbeg = (int64_t)blockIdx.y * rows_per;
-  const int64_t rend = imin(m, rbeg + rows_per);
-  S += (int64_t)blockIdx.y * split_stride;
-  float acc[VB][4];
-#pragma unroll
-  for (int v = 0; v < VB; ++v)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) acc[v][u] = 0.f;
-  constexpr int NC = RC * TN / 256, NX = RC * 16 * VB / 256;   // tile entries per thread
-  for (int64_t i0 = rbeg; i0 < rend; i0 += RC) {
-    // every load of the chunk in flight before the first store
-    float cl[NC], xl[NX];
-#pragma unroll
-    for (int u = 0; u < NC; ++u) {
-      const int e = threadIdx.x + 256 * u, r = e / TN, c = e % TN;
-      const int64_t gi = i0 + r, gc = col0 + c;
-      cl[u] = (gi < rend && gc < n) ? ld_elem(C, gi * n + gc) : 0.f;
-    }
-#pragma unroll
-    for (int u = 0; u < NX; ++u) {
-      const int e = threadIdx.x + 256 * u, r = e / (16 * VB), c = e % (16 * VB);
-      const int64_t gi = i0 + r;
-      xl[u] = (gi < rend && c < b) ? X[gi * ldx + c] : 0.f;
-    }
-#pragma unroll
-    for (int u = 0; u < NC; ++u) {
-      const int e = threadIdx.x + 256 * u;
-      Cs[e / TN][e % TN] = cl[u];
-    }
-#pragma unroll
-    for (int u = 0; u < NX; ++u) {
-      const int e = threadIdx.x + 256 * u;
-      Xs[e / (16 * VB)][e % (16 * VB)] = xl[u];
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int r = 0; r < RC; ++r) {
-      float cv[4], xv[VB];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) cv[u] = Cs[r][tx + 16 * u];
-#pragma unroll
-      for (int v = 0; v < VB; ++v) xv[v] = Xs[r][ty + 16 * v];
-#pragma unroll
-      for (int v = 0; v < VB; ++v)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[v][u] = fmaf(xv[v], cv[u], acc[v][u]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int v = 0; v < VB; ++v) {
-    int c = ty + 16 * v;
-    if (c >= b) continue;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      int64_t gc = col0 + tx + 16 * u;
-      if (gc < n) st_elem(S, (int64_t)c * lds + gc, acc[v][u]);
-    }
-  }
-}
+namespace {
 
 // ---------------------------------------------------------------- cs
-// P[split][i][c] = sum_{col in split} C[i][col] S[c][col] for the CTA's
-// 32-row tile; grid = (row tiles, splits).
-template <typename TIn, int VB>
-__global__ void __launch_bounds__(256) k_cs(const TIn* __restrict__ C, int64_t m, int64_t n,
-                                            const float* __restrict__ S, int64_t lds, int b,
-                                            float* __restrict__ P, int64_t cols_per_split) {
-  constexpr int TN = 64, RM = 32;
-  __shared__ float Cs[RM][TN + 1];
-  __shared__ float Ss[16 * VB][TN + 1];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int64_t row0 = (int64_t)blockIdx.x * RM;
-  const int64_t cbeg = (int64_t)blockIdx.y * cols_per_split;
-  const int64_t cend = min(n, cbeg + cols_per_split);
-  float acc[2][VB];
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int v = 0; v < VB; ++v) acc[a][v] = 0.f;
-  for (int64_t c0 = cbeg; c0 < cend; c0 += TN) {
-    for (int e = threadIdx.x; e < RM * TN; e += 256) {
-      int r = e / TN, c = e % TN;
-      int64_t gi = row0 + r, gc = c0 + c;
-      Cs[r][c] = (gi < m && gc < cend) ? ld_elem(C, gi * n + gc) : 0.f;
-    }
-    for (int e = threadIdx.x; e < 16 * VB * TN; e += 256) {
-      int r = e / TN, c = e % TN;
-      int64_t gc = c0 + c;
-      Ss[r][c] = (r < b && gc < cend) ? S[(int64_t)r * lds + gc] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int t = 0; t < TN; ++t) {
-      float ci[2], sv[VB];
-#pragma unroll
-      for (int a = 0; a < 2; ++a) ci[a] = Cs[ty + 16 * a][t];
-#pragma unroll
-      for (int v = 0; v < VB; ++v) sv[v] = Ss[tx + 16 * v][t];
-#pragma unroll
-      for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int v = 0; v < VB; ++v) acc[a][v] = fmaf(ci[a], sv[v], acc[a][v]);
-    }
-    __syncthreads();
-  }
-  float* out = P + (int64_t)blockIdx.y * m * b;
-#pragma unroll
-  for (int a = 0; a < 2; ++a) {
-    int64_t i = row0 + ty + 16 * a;
-    if (i >= m) continue;
-#pragma unroll
-    for (int v = 0; v < VB; ++v) {
-      int c = tx + 16 * v;
-      if (c < b) out[i * b + c] = acc[a][v];
-    }
-  }
-}
-
-// ---------------------------------------------------------------- ga (fused)
-// P[cta] = sum over the CTA's column tiles C_j (C_j^T X), m <= 256, b <= 48.
-// Each 32-column tile of C is loaded once into shared memory and used by both
-// products.  Accumulator rows i = ty + 16 a, columns c = tx + 16 v.
-template <typename TIn, int MA, int VB>
-__global__ void __launch_bounds__(256) k_ga_fused(const TIn* __restrict__ C, int64_t m, int64_t n,
-                                                  const float* __restrict__ X, int ldx, int b,
-                                                  float* __restrict__ P, int64_t tiles_per_cta) {
-  constexpr int TN = 32;
-  constexpr int MP = 16 * MA;            // padded row count
-  constexpr int BP = 16 * VB;            // padded column count
-  extern __shared__ float sm[];
-  float* Cs = sm;                        // [MP][TN + 1]
-  float* Xs = Cs + MP * (TN + 1);        // [MP][BP + 1]
-  float* Ts = Xs + MP * (BP + 1);        // [TN][BP + 1]
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  for (int e = threadIdx.x; e < MP * BP; e += 256) {
-    int r = e / BP, c = e % BP;
-    Xs[r * (BP + 1) + c] = (r < m && c < b) ? X[(int64_t)r * ldx + c] : 0.f;
-  }
-  float acc[MA][VB];
-#pragma unroll
-  for (int a = 0; a < MA; ++a)
-#pragma unroll
-    for (int v = 0; v < VB; ++v) acc[a][v] = 0.f;
-  const int64_t ntiles = (n + TN - 1) / TN;
-  const int64_t t_beg = (int64_t)blockIdx.x * tiles_per_cta;
-  const int64_t t_end = min(ntiles, t_beg + tiles_per_cta);
-  for (int64_t tile = t_beg; tile < t_end; ++tile) {
-    const int64_t c0 = tile * TN;
-    __syncthreads();
-    for (int e = threadIdx.x; e < MP * TN; e += 256) {
-      int r = e / TN, c = e % TN;
-      int64_t gc = c0 + c;
-      Cs[r * (TN + 1) + c] = (r < m && gc < n) ? ld_elem(C, (int64_t)r * n + gc) : 0.f;
-    }
-    __syncthreads();
-    // T[t][c] = sum_i C[i][t] X[i][c]; thread -> t = tx + 16 u (u < 2), c = ty + 16 v
-    {
-      float tacc[2][VB];
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < VB; ++v) tacc[u][v] = 0.f;
-      for (int i = 0; i < MP; ++i) {
-        float cv0 = Cs[i * (TN + 1) + tx], cv1 = Cs[i * (TN + 1) + tx + 16];
-#pragma unroll
-        for (int v = 0; v < VB; ++v) {
-          float xv = Xs[i * (BP + 1) + ty + 16 * v];
-          tacc[0][v] = fmaf(cv0, xv, tacc[0][v]);
-          tacc[1][v] = fmaf(cv1, xv, tacc[1][v]);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < VB; ++v) Ts[(tx + 16 * u) * (BP + 1) + ty + 16 * v] = tacc[u][v];
-    }
-    __syncthreads();
-    // acc[i][c] += sum_t C[i][t] T[t][c]
-#pragma unroll 4
-    for (int t = 0; t < TN; ++t) {
-      float tv[VB];
-#pragma unroll
-      for (int v = 0; v < VB; ++v) tv[v] = Ts[t * (BP + 1) + tx + 16 * v];
-#pragma unroll
-      for (int a = 0; a < MA; ++a) {
-        float cv = Cs[(ty + 16 * a) * (TN + 1) + t];
-#pragma unroll
-        for (int v = 0; v < VB; ++v) acc[a][v] = fmaf(cv, tv[v], acc[a][v]);
-      }
-    }
-  }
-  float* out = P + (int64_t)blockIdx.x * m * b;
-#pragma unroll
-  for (int a = 0; a < MA; ++a) {
-    int i = ty + 16 * a;
-    if (i >= m) continue;
-#pragma unroll
-    for (int v = 0; v < VB; ++v) {
-      int c = tx + 16 * v;
-      if (c < b) out[(int64_t)i * b + c] = acc[a][v];
-    }
-  }
+// P[split][i][c] = sum_{col in split} C[i][col] S[c][col], i in the CTA's
+// row tile; grid = (row tiles, splits).
+template <class Sh, typename TIn>
+__global__ void __launch_bounds__(256, 2) k_cs(const TIn* __restrict__ C, int64_t m, int64_t n,
+                                               const float* __restrict__ S, int64_t lds, int b,
+                                               float* __restrict__ P, int64_t cols_per_split, bool va, bool vb) {
+  extern __shared__ __align__(16) float nt_sm[];
+  const int64_t row0 = (int64_t)blockIdx.x * Sh::BM;
+  const int64_t cbeg = (int64_t)blockIdx.y * cols_per_split, cend = imin(n, cbeg + cols_per_split);
+  const int rows = (int)imin(Sh::BM, m - row0);
+  float* out = P + ((int64_t)blockIdx.y * m + row0) * b;
+  simt::nt_tile<Sh, false>(C + row0 * n, n, rows, S, lds, b, cbeg, cend, va, vb, nt_sm,
+                           [&](int i, int c, float s) {
+                             if (i < rows && c < b) out[(int64_t)i * b + c] = s;
+                           });
 }
 
 // ---------------------------------------------------------------- gram
-// P[cta] = sum over the CTA's column tiles C_j C_j^T, m <= 128.
-template <typename TIn, int MA>
-__global__ void __launch_bounds__(256) k_gram(const TIn* __restrict__ C, int64_t m, int64_t n,
-                                              float* __restrict__ P, int64_t tiles_per_cta) {
-  constexpr int TN = 32, MP = 16 * MA;
-  __shared__ float Cs[MP][TN + 1];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float acc[MA][MA];
+// P[item] (T x T, T = Sh::BM) = rows I of C times rows J of C, transposed,
+// over the item's column range; tiles I <= J enumerated J-major.
+template <class Sh, typename TIn>
+__global__ void __launch_bounds__(256, 2) k_gram_tiles_simt(const TIn* __restrict__ C, int64_t m, int64_t n, int splits,
+                                                            float* __restrict__ P, bool vec) {
+  extern __shared__ __align__(16) float nt_sm[];
+  constexpr int T = Sh::BM;
+  static_assert(Sh::BN == T, "square tiles");
+  const int t = (int)blockIdx.x / splits, s = (int)blockIdx.x % splits;
+  int J = 0;
+  while ((J + 1) * (J + 2) / 2 <= t) ++J;
+  const int I = t - J * (J + 1) / 2;
+  const int64_t chunks = ceil_div(n, Sh::BK);
+  const int64_t c0 = chunks * s / splits * Sh::BK, c1 = imin(n, chunks * (s + 1) / splits * Sh::BK);
+  const int ra = (int)imin(T, m - (int64_t)I * T), rb = (int)imin(T, m - (int64_t)J * T);
+  const TIn* A = C + (int64_t)I * T * n;
+  const TIn* B = C + (int64_t)J * T * n;
+  float* out = P + (size_t)blockIdx.x * T * T;
+  auto put = [&](int i, int c, float v) { out[i * T + c] = v; };
+  if (I == J) simt::nt_tile<Sh, true>(A, n, ra, A, n, ra, c0, c1, vec, vec, nt_sm, put);
+  else simt::nt_tile<Sh, false>(A, n, ra, B, n, rb, c0, c1, vec, vec, nt_sm, put);
+}
+
+// G[i][j] = G[j][i] = sum over the splits of tile(i, j), i <= j: eight warps
+// of a block take every eighth split of 32 consecutive j, in four chains, and
+// the warp sums are added in a fixed tree (one thread per entry left the
+// short Grams waiting on a chain of hundreds of loads).
+template <int T>
+__global__ void __launch_bounds__(256) k_gram_simt_reduce(const float* __restrict__ P, int64_t m, int splits,
+                                                          float* __restrict__ G) {
+  __shared__ float red[8][33];
+  const int i = blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int j = (int)blockIdx.x * 32 + lane;
+  if ((int)blockIdx.x * 32 + 31 < i) return;
+  const bool live = j >= i && j < m;
+  float a[4] = {0.f, 0.f, 0.f, 0.f};
+  if (live) {
+    const int I = i / T, J = j / T;
+    const int t = J * (J + 1) / 2 + I;
+    const float* src = P + (size_t)t * splits * T * T + (size_t)(i - T * I) * T + (j - T * J);
+    int k = w;
+    for (; k + 24 < splits; k += 32) {
 #pragma unroll
-  for (int a = 0; a < MA; ++a)
-#pragma unroll
-    for (int l = 0; l < MA; ++l) acc[a][l] = 0.f;
-  const int64_t ntiles = (n + TN - 1) / TN;
-  const int64_t t_beg = (int64_t)blockIdx.x * tiles_per_cta;
-  const int64_t t_end = min(ntiles, t_beg + tiles_per_cta);
-  for (int64_t tile = t_beg; tile < t_end; ++tile) {
-    const int64_t c0 = tile * TN;
-    __syncthreads();
-    for (int e = threadIdx.x; e < MP * TN; e += 256) {
-      int r = e / TN, c = e % TN;
-      int64_t gc = c0 + c;
-      Cs[r][c] = (r < m && gc < n) ? ld_elem(C, (int64_t)r * n + gc) : 0.f;
+      for (int u = 0; u < 4; ++u) a[u] += src[(size_t)(k + 8 * u) * T * T];
     }
-    __syncthreads();
-#pragma unroll 4
-    for (int t = 0; t < TN; ++t) {
-      float ci[MA], cj[MA];
-#pragma unroll
-      for (int a = 0; a < MA; ++a) ci[a] = Cs[ty + 16 * a][t];
-#pragma unroll
-      for (int l = 0; l < MA; ++l) cj[l] = Cs[tx + 16 * l][t];
-#pragma unroll
-      for (int a = 0; a < MA; ++a)
-#pragma unroll
-        for (int l = 0; l < MA; ++l) acc[a][l] = fmaf(ci[a], cj[l], acc[a][l]);
-    }
+    for (; k < splits; k += 8) a[0] += src[(size_t)k * T * T];
   }
-  float* out = P + (int64_t)blockIdx.x * m * m;
-#pragma unroll
-  for (int a = 0; a < MA; ++a) {
-    int i = ty + 16 * a;
-    if (i >= m) continue;
-#pragma unroll
-    for (int l = 0; l < MA; ++l) {
-      int j = tx + 16 * l;
-      if (j < m) out[(int64_t)i * m + j] = acc[a][l];
-    }
+  red[w][lane] = (a[0] + a[1]) + (a[2] + a[3]);
+  __syncthreads();
+  if (w == 0 && live) {
+    const float s = ((red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane])) +
+                    ((red[4][lane] + red[5][lane]) + (red[6][lane] + red[7][lane]));
+    G[(int64_t)i * m + j] = s;
+    if (j != i) G[(int64_t)j * m + i] = s;
   }
 }
 
@@ -352,11 +163,11 @@ __global__ void __launch_bounds__(32 * RED_WARPS) k_reduce_grouped(const float* 
   reduce_elements(PartialsGrouped{P, E, cols, group_rows}, per, (int64_t)groups * E, E, cols, out, ldo);
 }
 
+}  // namespace
+
 // ======================================================================
 // Launchers
 // ======================================================================
-static int target_ctas() { return 4 * 152; }
-
 static void reduce_launch(const float* P, int S, int64_t rows, int cols, float* out, int64_t ldo,
                           cudaStream_t st) {
   int64_t E = rows * cols;
@@ -380,225 +191,128 @@ cudaError_t launch_reduce_partials_grouped(const float* P, int per, int groups, 
   return cudaGetLastError();
 }
 
-// S (b x n) = sum over row splits of the partials P[y] (b x n), fixed order.
-template <typename TOut>
-__global__ void k_sum_splits(const float* __restrict__ P, int splits, int b, int64_t n, TOut* __restrict__ S,
-                             int64_t lds) {
-  const int64_t E = (int64_t)b * n;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x) {
-    // eight loads in flight, added in split order
-    float acc = 0.f;
-    int y = 0;
-    for (; y + 8 <= splits; y += 8) {
-      float v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = P[(int64_t)(y + u) * E + e];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) acc += v[u];
-    }
-    for (; y < splits; ++y) acc += P[(int64_t)y * E + e];
-    st_elem(S, (e / n) * lds + e % n, acc);
-  }
+namespace {
+
+// Rows of a cs tile: the shortest of 32, 48 and 64 that needs no more tiles.
+int cs_tile_rows(int64_t m) { return m <= 32 ? 32 : m <= 48 ? 48 : 64; }
+
+// Two CTAs an SM in all, a split at least 256 columns.
+int64_t cs_splits(int64_t m, int64_t n) {
+  const int64_t rt = ceil_div(m, cs_tile_rows(m));
+  return imax(1, imin(imax(1, 2 * 152 / rt), ceil_div(n, 256)));
 }
 
-// Row splits of the tall-thin form: 32 rows (one tile chunk) per CTA, at most
-// 64 splits.
-int64_t simt_proj_splits(int64_t m, int64_t n) {
-  if (n > 512 || m < 256) return 1;
-  return imin(ceil_div(m, 32), 64);
-}
-
-template <typename TIn, typename TOut>
-cudaError_t simt_proj(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b, TOut* S,
-                      int64_t lds, cudaStream_t st, float* partials) {
-  const int64_t splits = partials ? simt_proj_splits(m, n) : 1;
-  if (splits > 1) {
-    // tall-thin unfolding: rows split across CTAs, then a fixed-order sum
-    const int64_t rows_per = ceil_div(m, splits);
-    dim3 grid((unsigned)ceil_div(n, 64), (unsigned)splits);
-    ProfScope prof("proj_simt", st, (double)m * n * sizeof(TIn) + (double)m * b * 4 + (double)b * n * sizeof(TOut),
-                   2.0 * m * n * b);
-    note_launch("proj_simt", 2);
-#define TTR_PS(VB) k_proj<TIn, float, VB><<<grid, 256, 0, st>>>(C, m, n, X, ldx, b, partials, n, rows_per, (int64_t)b * n)
-    if (b <= 16) TTR_PS(1); else if (b <= 32) TTR_PS(2); else if (b <= 48) TTR_PS(3); else if (b <= 64) TTR_PS(4);
-    else return cudaErrorInvalidValue;
-#undef TTR_PS
-    const int64_t E = (int64_t)b * n;
-    k_sum_splits<TOut><<<(int)imin(ceil_div(E, 256), 256), 256, 0, st>>>(partials, (int)splits, b, n, S, lds);
-    return cudaGetLastError();
+template <class Sh, typename TIn>
+cudaError_t cs_launch(const TIn* C, int64_t m, int64_t n, const float* S, int64_t lds, int b, float* P, int splits,
+                      cudaStream_t st) {
+  const int64_t per = ceil_div(ceil_div(n, Sh::BK), splits) * Sh::BK;
+  constexpr size_t smem = sizeof(float) * Sh::smem_floats(false);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = raise_smem_limit(k_cs<Sh, TIn>);
+    if (e != cudaSuccess) return e;
   }
-  dim3 grid((unsigned)ceil_div(n, 64));
-  ProfScope prof("proj_simt", st, (double)m * n * sizeof(TIn) + (double)m * b * 4 + (double)b * n * sizeof(TOut),
-                 2.0 * m * n * b);
-  note_launch("proj_simt");
-  if (b <= 16)
-    k_proj<TIn, TOut, 1><<<grid, 256, 0, st>>>(C, m, n, X, ldx, b, S, lds, m, 0);
-  else if (b <= 32)
-    k_proj<TIn, TOut, 2><<<grid, 256, 0, st>>>(C, m, n, X, ldx, b, S, lds, m, 0);
-  else if (b <= 48)
-    k_proj<TIn, TOut, 3><<<grid, 256, 0, st>>>(C, m, n, X, ldx, b, S, lds, m, 0);
-  else if (b <= 64)
-    k_proj<TIn, TOut, 4><<<grid, 256, 0, st>>>(C, m, n, X, ldx, b, S, lds, m, 0);
-  else
-    return cudaErrorInvalidValue;
+  k_cs<Sh, TIn><<<dim3((unsigned)ceil_div(m, Sh::BM), (unsigned)splits), 256, smem, st>>>(
+      C, m, n, S, lds, b, P, per, simt::rows_aligned4(C, n), simt::rows_aligned4(S, lds));
   return cudaGetLastError();
 }
 
-int64_t simt_cs_splits(int64_t m, int64_t n) {
-  int64_t rt = ceil_div(m, 32);
-  int64_t s = imax(1, target_ctas() / rt);
-  s = imin(s, imax(1, ceil_div(n, 256)));
-  return s;
+template <int TR, typename TIn>
+cudaError_t cs_dispatch(const TIn* C, int64_t m, int64_t n, const float* S, int64_t lds, int b, float* P, int splits,
+                        cudaStream_t st) {
+#define TTR_CS(TC, CT) return cs_launch<simt::NtShape<TR, TC, CT>>(C, m, n, S, lds, b, P, splits, st)
+  if (b <= 4) TTR_CS(4, 1);
+  if (b <= 6) TTR_CS(6, 1);
+  if (b <= 8) TTR_CS(8, 1);
+  if (b <= 12) TTR_CS(6, 2);
+  if (b <= 16) TTR_CS(8, 2);
+  if (b <= 20) TTR_CS(5, 4);
+  if (b <= 24) TTR_CS(6, 4);
+  if (b <= 32) TTR_CS(8, 4);
+  if (b <= 40) TTR_CS(5, 8);
+  if (b <= 48) TTR_CS(6, 8);
+  if (b <= 64) TTR_CS(8, 8);
+#undef TTR_CS
+  return cudaErrorInvalidValue;
 }
+
+}  // namespace
 
 template <typename TIn>
 cudaError_t simt_cs(const TIn* C, int64_t m, int64_t n, const float* S, int64_t lds, int b,
                     float* partials, float* out, int64_t ldo, cudaStream_t st) {
-  int64_t splits = simt_cs_splits(m, n);
-  int64_t per = ceil_div(ceil_div(n, 64), splits) * 64;
-  dim3 grid((unsigned)ceil_div(m, 32), (unsigned)splits);
+  const int splits = (int)cs_splits(m, n);
   {
-  ProfScope prof("cs_simt", st, (double)m * n * sizeof(TIn) + (double)b * n * 4, 2.0 * m * n * b);
-  note_launch("cs_simt");
-  if (b <= 16)
-    k_cs<TIn, 1><<<grid, 256, 0, st>>>(C, m, n, S, lds, b, partials, per);
-  else if (b <= 32)
-    k_cs<TIn, 2><<<grid, 256, 0, st>>>(C, m, n, S, lds, b, partials, per);
-  else if (b <= 48)
-    k_cs<TIn, 3><<<grid, 256, 0, st>>>(C, m, n, S, lds, b, partials, per);
-  else if (b <= 64)
-    k_cs<TIn, 4><<<grid, 256, 0, st>>>(C, m, n, S, lds, b, partials, per);
-  else
-    return cudaErrorInvalidValue;
+    ProfScope prof("cs_simt", st, (double)m * n * sizeof(TIn) + (double)b * n * 4, 2.0 * m * n * b);
+    note_launch("cs_simt");
+    const int rows = cs_tile_rows(m);
+    const cudaError_t e = rows == 32   ? cs_dispatch<4>(C, m, n, S, lds, b, partials, splits, st)
+                          : rows == 48 ? cs_dispatch<6>(C, m, n, S, lds, b, partials, splits, st)
+                                       : cs_dispatch<8>(C, m, n, S, lds, b, partials, splits, st);
+    if (e != cudaSuccess) return e;
   }
-  reduce_launch(partials, (int)splits, m, b, out, ldo, st);
+  reduce_launch(partials, splits, m, b, out, ldo, st);
   return cudaGetLastError();
 }
 
-int64_t simt_tiles_split(int64_t n, int64_t tn) {
-  int64_t tiles = ceil_div(n, tn);
-  int64_t ctas = imin(tiles, target_ctas());
-  return ceil_div(tiles, ctas);   // tiles per CTA
+int64_t simt_cs_partials(int64_t m, int64_t n, int b) { return cs_splits(m, n) * m * b; }
+
+// ---------------------------------------------------------------- gram
+namespace {
+
+int gram_tile(int64_t m) { return m <= 16 ? 16 : m <= 32 ? 32 : m <= 48 ? 48 : 64; }
+
+// Tiles of the upper triangle and splits of the columns: two CTAs an SM, a
+// split at least 256 columns.
+void gram_plan(int64_t m, int64_t n, int* tiles, int* splits) {
+  const int nT = (int)ceil_div(m, gram_tile(m));
+  *tiles = nT * (nT + 1) / 2;
+  *splits = (int)imax(1, imin(2 * 152 / *tiles, ceil_div(n, 256)));
 }
 
-template <typename TIn, int MA, int VB>
-static void ga_launch(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b, float* P,
-                      int64_t tpc, int ctas, cudaStream_t st) {
-  size_t smem = sizeof(float) * ((16 * MA) * 33 + (16 * MA) * (16 * VB + 1) + 32 * (16 * VB + 1));
-  auto kern = k_ga_fused<TIn, MA, VB>;
-  raise_smem_limit(kern);
-  kern<<<ctas, 256, smem, st>>>(C, m, n, X, ldx, b, P, tpc);
-}
-
-template <typename TIn, int VB>
-static cudaError_t ga_dispatch_m(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b,
-                                 float* P, int64_t tpc, int ctas, cudaStream_t st) {
-  int ma = (int)ceil_div(m, 16);
-  switch (ma) {
-#define TTR_GA_CASE(K) \
-  case K: ga_launch<TIn, K, VB>(C, m, n, X, ldx, b, P, tpc, ctas, st); break;
-    TTR_GA_CASE(1) TTR_GA_CASE(2) TTR_GA_CASE(3) TTR_GA_CASE(4) TTR_GA_CASE(5) TTR_GA_CASE(6)
-    TTR_GA_CASE(7) TTR_GA_CASE(8) TTR_GA_CASE(9) TTR_GA_CASE(10) TTR_GA_CASE(11) TTR_GA_CASE(12)
-    TTR_GA_CASE(13) TTR_GA_CASE(14) TTR_GA_CASE(15) TTR_GA_CASE(16)
-#undef TTR_GA_CASE
-    default: return cudaErrorInvalidValue;
+template <class Sh, typename TIn>
+cudaError_t gram_launch(const TIn* C, int64_t m, int64_t n, int tiles, int splits, float* P, float* G,
+                        cudaStream_t st) {
+  constexpr size_t smem = sizeof(float) * Sh::smem_floats(false);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = raise_smem_limit(k_gram_tiles_simt<Sh, TIn>);
+    if (e != cudaSuccess) return e;
   }
-  return cudaSuccess;
+  k_gram_tiles_simt<Sh, TIn><<<tiles * splits, 256, smem, st>>>(C, m, n, splits, P, simt::rows_aligned4(C, n));
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  note_launch("gram_reduce");
+  k_gram_simt_reduce<Sh::BM><<<dim3((unsigned)ceil_div(m, 32), (unsigned)m), 256, 0, st>>>(P, m, splits, G);
+  return cudaGetLastError();
 }
 
-bool simt_ga_fused_ok(int64_t m, int b) { return m <= 256 && b <= 48 && ceil_div(m, 16) * ceil_div(b, 16) <= 48; }
+}  // namespace
 
 template <typename TIn>
-cudaError_t simt_ga(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b,
-                    float* partials, float* out, int64_t ldo, cudaStream_t st) {
-  if (!simt_ga_fused_ok(m, b)) return cudaErrorInvalidValue;
-  int64_t tpc = simt_tiles_split(n, 32);
-  int ctas = (int)ceil_div(ceil_div(n, 32), tpc);
-  cudaError_t e;
-  {
-  ProfScope prof("gram_apply_simt", st, (double)m * n * sizeof(TIn) + (double)m * b * 4, 4.0 * m * n * b);
-  note_launch("gram_apply_simt");
-  if (b <= 16)
-    e = ga_dispatch_m<TIn, 1>(C, m, n, X, ldx, b, partials, tpc, ctas, st);
-  else if (b <= 32)
-    e = ga_dispatch_m<TIn, 2>(C, m, n, X, ldx, b, partials, tpc, ctas, st);
-  else
-    e = ga_dispatch_m<TIn, 3>(C, m, n, X, ldx, b, partials, tpc, ctas, st);
+cudaError_t simt_gram(const TIn* C, int64_t m, int64_t n, float* partials, float* out, cudaStream_t st,
+                      const char* family) {
+  int tiles, splits;
+  gram_plan(m, n, &tiles, &splits);
+  ProfScope prof(family, st, (double)m * n * sizeof(TIn), 2.0 * m * m * n);
+  note_launch(family);
+  switch (gram_tile(m)) {
+    case 16: return gram_launch<simt::NtShape<2, 8, 2>>(C, m, n, tiles, splits, partials, out, st);
+    case 32: return gram_launch<simt::NtShape<4, 8, 4>>(C, m, n, tiles, splits, partials, out, st);
+    case 48: return gram_launch<simt::NtShape<6, 6, 8>>(C, m, n, tiles, splits, partials, out, st);
+    default: return gram_launch<simt::NtShape<8, 8, 8>>(C, m, n, tiles, splits, partials, out, st);
   }
-  if (e != cudaSuccess) return e;
-  reduce_launch(partials, ctas, m, b, out, ldo, st);
-  return cudaGetLastError();
 }
 
-// Fused Gram-apply with at most max_ctas CTAs, so that the partials fit a
-// caller-given buffer of max_ctas * m * b floats.
-template <typename TIn>
-cudaError_t simt_ga_with_ctas(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b,
-                              float* partials, int64_t max_ctas, float* out, int64_t ldo, cudaStream_t st) {
-  if (!simt_ga_fused_ok(m, b) || max_ctas < 1) return cudaErrorInvalidValue;
-  const int64_t tiles = ceil_div(n, 32);
-  const int64_t ctas0 = imin(imin(tiles, target_ctas()), max_ctas);
-  const int64_t tpc = ceil_div(tiles, ctas0);
-  const int ctas = (int)ceil_div(tiles, tpc);
-  cudaError_t e;
-  {
-    ProfScope prof("gram_apply_simt", st, (double)m * n * sizeof(TIn) + (double)m * b * 4, 4.0 * m * n * b);
-    note_launch("gram_apply_simt");
-    if (b <= 16)
-      e = ga_dispatch_m<TIn, 1>(C, m, n, X, ldx, b, partials, tpc, ctas, st);
-    else if (b <= 32)
-      e = ga_dispatch_m<TIn, 2>(C, m, n, X, ldx, b, partials, tpc, ctas, st);
-    else
-      e = ga_dispatch_m<TIn, 3>(C, m, n, X, ldx, b, partials, tpc, ctas, st);
-  }
-  if (e != cudaSuccess) return e;
-  reduce_launch(partials, ctas, m, b, out, ldo, st);
-  return cudaGetLastError();
-}
-template cudaError_t simt_ga_with_ctas<float>(const float*, int64_t, int64_t, const float*, int, int, float*, int64_t, float*, int64_t, cudaStream_t);
-template cudaError_t simt_ga_with_ctas<__nv_bfloat16>(const __nv_bfloat16*, int64_t, int64_t, const float*, int, int, float*, int64_t, float*, int64_t, cudaStream_t);
-
-int64_t simt_ga_partials(int64_t m, int64_t n, int b) {
-  int64_t tpc = simt_tiles_split(n, 32);
-  return ceil_div(ceil_div(n, 32), tpc) * m * b;
-}
-int64_t simt_cs_partials(int64_t m, int64_t n, int b) { return simt_cs_splits(m, n) * m * b; }
 int64_t simt_gram_partials(int64_t m, int64_t n) {
-  int64_t tpc = simt_tiles_split(n, 32);
-  return ceil_div(ceil_div(n, 32), tpc) * m * m;
-}
-
-template <typename TIn>
-cudaError_t simt_gram(const TIn* C, int64_t m, int64_t n, float* partials, float* out, cudaStream_t st) {
-  int64_t tpc = simt_tiles_split(n, 32);
-  int ctas = (int)ceil_div(ceil_div(n, 32), tpc);
-  int ma = (int)ceil_div(m, 16);
-  {
-  ProfScope prof("gram_simt", st, (double)m * n * sizeof(TIn), 2.0 * m * m * n);
-  note_launch("gram_simt");
-  switch (ma) {
-#define TTR_GR_CASE(K) \
-  case K: k_gram<TIn, K><<<ctas, 256, 0, st>>>(C, m, n, partials, tpc); break;
-    TTR_GR_CASE(1) TTR_GR_CASE(2) TTR_GR_CASE(3) TTR_GR_CASE(4) TTR_GR_CASE(5) TTR_GR_CASE(6)
-    TTR_GR_CASE(7) TTR_GR_CASE(8)
-#undef TTR_GR_CASE
-    default: return cudaErrorInvalidValue;
-  }
-  }
-  reduce_launch(partials, ctas, m, (int)m, out, m, st);
-  return cudaGetLastError();
+  int tiles, splits;
+  gram_plan(m, n, &tiles, &splits);
+  const int64_t t = gram_tile(m);
+  return (int64_t)tiles * splits * t * t;
 }
 
 // Explicit instantiations.
-template cudaError_t simt_proj<float, float>(const float*, int64_t, int64_t, const float*, int, int, float*, int64_t, cudaStream_t, float*);
-template cudaError_t simt_proj<float, __nv_bfloat16>(const float*, int64_t, int64_t, const float*, int, int, __nv_bfloat16*, int64_t, cudaStream_t, float*);
-template cudaError_t simt_proj<__nv_bfloat16, float>(const __nv_bfloat16*, int64_t, int64_t, const float*, int, int, float*, int64_t, cudaStream_t, float*);
-template cudaError_t simt_proj<__nv_bfloat16, __nv_bfloat16>(const __nv_bfloat16*, int64_t, int64_t, const float*, int, int, __nv_bfloat16*, int64_t, cudaStream_t, float*);
 template cudaError_t simt_cs<float>(const float*, int64_t, int64_t, const float*, int64_t, int, float*, float*, int64_t, cudaStream_t);
 template cudaError_t simt_cs<__nv_bfloat16>(const __nv_bfloat16*, int64_t, int64_t, const float*, int64_t, int, float*, float*, int64_t, cudaStream_t);
-template cudaError_t simt_ga<float>(const float*, int64_t, int64_t, const float*, int, int, float*, float*, int64_t, cudaStream_t);
-template cudaError_t simt_ga<__nv_bfloat16>(const __nv_bfloat16*, int64_t, int64_t, const float*, int, int, float*, float*, int64_t, cudaStream_t);
-template cudaError_t simt_gram<float>(const float*, int64_t, int64_t, float*, float*, cudaStream_t);
-template cudaError_t simt_gram<__nv_bfloat16>(const __nv_bfloat16*, int64_t, int64_t, float*, float*, cudaStream_t);
+template cudaError_t simt_gram<float>(const float*, int64_t, int64_t, float*, float*, cudaStream_t, const char*);
+template cudaError_t simt_gram<__nv_bfloat16>(const __nv_bfloat16*, int64_t, int64_t, float*, float*, cudaStream_t, const char*);
 
 }  // namespace ttr

@@ -52,122 +52,181 @@ __device__ inline void chol_inv_cta(float* G, int ldg, int b, const float* diag0
 }
 
 
-// Cholesky factorisation and triangular inverse of a b x b Gram, b <= 32,
-// by one warp (the calling warp, all 32 lanes; one warp of a CTA at a time,
-// since the routine keeps its rows of R in static shared arrays), in one
-// sweep.  Lane l holds column l of the upper triangle of G in a register
-// window that slides down one row per step: at step j, a[s] = G[j + s][l],
-// so the pivot row is always a[0] and every register index is a
-// compile-time constant while the column loop runs at run time.  Row j of
-// R goes to R and, shifted so that it starts at R[j][j + 1], to a
-// 16-byte-aligned shared row Rs[j], which every lane reads back as eight
-// vector broadcasts.  The same row updates row l of V (started as the
-// identity), held as the window v[s] = V[l][j + s]: T[l][j] = V[l][j] /
-// R[j][j] is final at step j, and V[l][j + s] -= R[j][j + s] T[l][j]
-// (T[:, c] = (e_c - sum_{j < c} R[j][c] T[:, j]) / R[c][c], i.e. T R = I),
-// so no triangular solve follows.  T is staged transposed (conflict-free)
-// and written row by row at the end.  Entries past row or column b are
-// exact zeros in Rs and in the windows, so the sums run over full vectors
-// without changing a bit of the result.  Pivot square roots and
-// reciprocals use the hardware reciprocal square root (a few ulp), which
-// the following Cholesky QR passes absorb.  A pivot below 1e-6 of diag0
-// (or non-positive) raises *flag when report and is replaced by 1.
-// Callers use the out-of-line copy below.
-__device__ __forceinline__ void chol_inv_warp(const float* G, int ldg, int b, const float* diag0, float* R,
-                                                   int ldr, float* T, int ldt, int* flag, bool report,
-                                                   unsigned long long* badmask, int bit0 = 0) {
-  __shared__ __align__(16) float Rs[32][36];   // Rs[j][s] = R[j][j + 1 + s], zero past column b
-  __shared__ float Tt[32][33];                 // Tt[j][l] = T[l][j]
+// Cholesky factorisation G = R^T R and the triangular inverse T = R^-1 of a
+// b x b Gram, b <= W (W = 16 or 32), by the first two warps of the CTA, both
+// in one sweep over the columns (no triangular solve follows).
+//
+// Warp 0 factors.  Lane l holds column l of the upper triangle of G in a
+// register window that slides down one row per step: at step j,
+// a[s] = G[j + s][l], so the pivot row is always a[0] and every register
+// index is a compile-time constant while the column loop runs at run time.
+// Row j of R, shifted so that it starts at R[j][j + 1], goes to a
+// 16-byte-aligned shared row, which every lane reads back as W / 4 vector
+// broadcasts to update its window.  The next pivot needs only lane j + 1's own
+// entries (G[j+1][j+1] - R[j][j+1]^2, the product the window update forms),
+// so its broadcast and reciprocal square root run while the row travels.
+// Warp 1 inverts, up to four rows behind (named barriers 1 .. 8, one per four
+// rows: warp 0 arrives, warp 1 waits).  Lane l holds row l of V, started as
+// the identity, as the window v[s] = V[l][j + s]: T[l][j] = V[l][j] / R[j][j]
+// is final at step j, and V[l][j + s] -= R[j][j + s] T[l][j]
+// (T[:, c] = (e_c - sum_{j < c} R[j][c] T[:, j]) / R[c][c], i.e. T R = I).
+// T is staged transposed (conflict-free) and written by the whole CTA.
+// Entries past row or column b are exact zeros in the shared rows and in the
+// windows, so the sums run over full vectors without changing a bit of the
+// result.  Pivot square roots and reciprocals use the hardware reciprocal
+// square root (a few ulp), which the following Cholesky QR passes absorb.  A
+// pivot below 1e-6 of diag0 (or non-positive) raises *flag when report and
+// is replaced by 1.
+//
+// The step's latency decides the time, and one warp doing both sweeps in
+// turn pays it twice: b = 30 took 15.1K cycles on one warp, 7.7K on two
+// (bit-identical).
+template <int W>
+struct CholShared {
+  float rows[W][W];      // rows[j][s] = R[j][j + 1 + s], zero past column b
+  float inv[W];          // 1 / R[j][j]
+  float Tt[W][33];       // Tt[j][l] = T[l][j]
+};
+
+template <int W>
+__device__ __forceinline__ void chol_warp(CholShared<W>& sh, const float* G, int ldg, int b, const float* diag0,
+                                          int* flag, bool report, unsigned long long* badmask, int bit0) {
   const unsigned full = 0xffffffffu;
   const int l = threadIdx.x & 31;
+  float a[W];
 #pragma unroll
-  for (int q = 0; q < 32; ++q) Rs[q][l] = 0.f;
-  if (l < 4) {
-#pragma unroll
-    for (int q = 0; q < 32; ++q) Rs[q][32 + l] = 0.f;
-  }
-  float a[32];                            // a[s] = G[j + s][l] at step j (rows <= l)
-  float v[32];                            // v[s] = V[l][j + s] at step j
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    a[i] = (i <= l && l < b) ? G[i * ldg + l] : 0.f;
-    v[i] = (i == l && l < b) ? 1.f : 0.f;
-  }
+  for (int i = 0; i < W; ++i) a[i] = (i <= l && l < b) ? G[i * ldg + l] : 0.f;
   const float d0 = (l < b) ? diag0[l] : 1.f;
-  bool bad = false;
-  unsigned long long badbits = 0ull;
-  __syncwarp();
+  float djj = __shfl_sync(full, a[0], 0);
+  const float dref0 = __shfl_sync(full, d0, 0);
+  bool low = !(djj > 1e-6f * dref0);
+  unsigned bad = low ? 1u : 0u;
+  djj = low ? 1.f : djj;
+  float inv = rsqrtf(djj);
 #pragma unroll 1
   for (int j = 0; j < b; ++j) {
-    float djj = __shfl_sync(full, a[0], j);
-    const float dref = __shfl_sync(full, d0, j);
-    if (!(djj > 1e-6f * dref)) {
-      bad = true;
-      badbits |= 1ull << j;
-      djj = 1.f;
-    }
-    const float inv = rsqrtf(djj);
-    const float rjl = (l == j) ? djj * inv : ((l > j) ? a[0] * inv : 0.f);   // R[j][l]
-    const float tlj = v[0] * inv;                                            // T[l][j]
-    if (l < b) R[j * ldr + l] = rjl;
-    if (l > j) Rs[j][l - j - 1] = rjl;
-    Tt[j][l] = tlj;
+    const float rjl = (l > j) ? a[0] * inv : ((l == j) ? djj * inv : 0.f);   // R[j][l]
+    // lane l > j holds entry l - j - 1; the others zero the rest of the row
+    if (l < W) sh.rows[j][l > j ? l - j - 1 : W - 1 - l] = (l > j) ? rjl : 0.f;
+    if (l == 0) sh.inv[j] = inv;
     __syncwarp();
-    // G[j + s][l] -= R[j][j + s] R[j][l] and V[l][j + s] -= R[j][j + s] T[l][j],
-    // then slide both windows down a row
-    const float4* rv = reinterpret_cast<const float4*>(Rs[j]);
+    const int nx = (j + 1) & 31;
+    const float cand = __shfl_sync(full, fmaf(-rjl, rjl, a[1]), nx);
+    const float dref = __shfl_sync(full, d0, nx);
+    const float4* rv = reinterpret_cast<const float4*>(sh.rows[j]);
+    float4 r4[W / 4];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const float4 r4 = rv[q];
-      const float rr[4] = {r4.x, r4.y, r4.z, r4.w};
+    for (int q = 0; q < W / 4; ++q) r4[q] = rv[q];
+    // issue is in order: the next pivot before the window update, so that it
+    // fills the wait for the row and its square root runs under the update
+    low = !(cand > 1e-6f * dref);
+    bad |= (low && j + 1 < b) ? (1u << nx) : 0u;
+    djj = low ? 1.f : cand;
+    inv = rsqrtf(djj);
+#pragma unroll
+    for (int q = 0; q < W / 4; ++q) {
+      const float rr[4] = {r4[q].x, r4[q].y, r4[q].z, r4[q].w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int s = 4 * q + e + 1;
-        if (s < 32) {
-          a[s - 1] = fmaf(-rr[e], rjl, a[s]);
-          v[s - 1] = fmaf(-rr[e], tlj, v[s]);
-        }
+        if (s < W) a[s - 1] = fmaf(-rr[e], rjl, a[s]);   // G[j + s][l] -= R[j][j + s] R[j][l], slid down a row
       }
     }
-    a[31] = 0.f;
-    v[31] = 0.f;
+    a[W - 1] = 0.f;
+    if ((j & 3) == 3 || j == b - 1)
+      asm volatile("bar.arrive %0, 64;\n" ::"r"(1 + (j >> 2)) : "memory");
   }
   if (report && bad && l == 0 && flag) atomicExch(flag, 1);
-  if (badmask && badbits && l == 0) atomicOr(badmask, badbits << bit0);
-  __syncwarp();
-  // row r of T: lane l writes T[r][l] = Tt[l][r] (zero below the diagonal)
-  for (int r = 0; r < b; ++r)
-    if (l < b) T[r * ldt + l] = (l >= r) ? Tt[l][r] : 0.f;
-  __syncwarp();
+  if (badmask && bad && l == 0) atomicOr(badmask, (unsigned long long)bad << bit0);
 }
 
-// Out-of-line copy (one per kernel, its own register allocation).
-static __device__ __noinline__ void chol_inv_warp_ool(const float* G, int ldg, int b, const float* diag0, float* R,
-                                                       int ldr, float* T, int ldt, int* flag, bool report,
-                                                       unsigned long long* badmask, int bit0) {
-  chol_inv_warp(G, ldg, b, diag0, R, ldr, T, ldt, flag, report, badmask, bit0);
+template <int W>
+__device__ __forceinline__ void inv_warp(CholShared<W>& sh, int b) {
+  const int l = threadIdx.x & 31;
+  float v[W];
+#pragma unroll
+  for (int i = 0; i < W; ++i) v[i] = (i == l && l < b) ? 1.f : 0.f;
+#pragma unroll 1
+  for (int j = 0; j < b; ++j) {
+    if ((j & 3) == 0) asm volatile("bar.sync %0, 64;\n" ::"r"(1 + (j >> 2)) : "memory");
+    const float4* rv = reinterpret_cast<const float4*>(sh.rows[j]);
+    const float inv = sh.inv[j];
+    float4 r4[W / 4];
+#pragma unroll
+    for (int q = 0; q < W / 4; ++q) r4[q] = rv[q];
+    const float t = v[0] * inv;                          // T[l][j]
+#pragma unroll
+    for (int q = 0; q < W / 4; ++q) {
+      const float rr[4] = {r4[q].x, r4[q].y, r4[q].z, r4[q].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int s = 4 * q + e + 1;
+        if (s < W) v[s - 1] = fmaf(-rr[e], t, v[s]);
+      }
+    }
+    v[W - 1] = 0.f;
+    sh.Tt[j][l] = t;
+  }
 }
 
-// chol_inv_cta's contract for b <= 32: the CTA synchronises, warp 0 alone
-// factors (the other warps do not enter the call), the CTA synchronises.
-__device__ __forceinline__ void chol_inv_warp32_call(const float* G, int ldg, int b, const float* diag0, float* R,
-                                                     int ldr, float* T, int ldt, int* flag, bool report,
+// One per kernel and width.
+template <int W>
+__device__ __forceinline__ CholShared<W>& chol_shared() {
+  __shared__ __align__(16) CholShared<W> sh;
+  return sh;
+}
+
+// Out of line (one copy per kernel, its own register allocation).
+template <int W>
+static __device__ __noinline__ void chol_inv_pair(CholShared<W>& sh, const float* G, int ldg, int b,
+                                                  const float* diag0, int* flag, bool report,
+                                                  unsigned long long* badmask, int bit0) {
+  if (threadIdx.x < 32) chol_warp<W>(sh, G, ldg, b, diag0, flag, report, badmask, bit0);
+  else inv_warp<W>(sh, b);
+}
+
+// Called by every thread of the CTA after a barrier: warps 0 and 1 work, then
+// all threads write T (zero below the diagonal); no barrier at the end.
+template <int W>
+static __device__ __forceinline__ void chol_inv_cta_w(const float* G, int ldg, int b, const float* diag0, float* T,
+                                                      int ldt, int* flag, bool report, unsigned long long* badmask,
+                                                      int bit0) {
+  CholShared<W>& sh = chol_shared<W>();
+  if (threadIdx.x < 64) chol_inv_pair<W>(sh, G, ldg, b, diag0, flag, report, badmask, bit0);
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  if (lane < b)
+    for (int r = threadIdx.x >> 5; r < b; r += blockDim.x >> 5)
+      T[r * ldt + lane] = (lane >= r) ? sh.Tt[lane][r] : 0.f;
+}
+static __device__ __forceinline__ void chol_inv_two_warps(const float* G, int ldg, int b, const float* diag0, float* T,
+                                                          int ldt, int* flag, bool report,
+                                                          unsigned long long* badmask, int bit0) {
+  if (b <= 16) chol_inv_cta_w<16>(G, ldg, b, diag0, T, ldt, flag, report, badmask, bit0);
+  else chol_inv_cta_w<32>(G, ldg, b, diag0, T, ldt, flag, report, badmask, bit0);
+}
+
+// chol_inv_cta's contract for b <= 32 in a CTA of at least two warps, except
+// that R itself is not written: the CTA synchronises, warps 0 and 1 factor and
+// invert, the CTA synchronises.
+__device__ __forceinline__ void chol_inv_warp32_call(const float* G, int ldg, int b, const float* diag0, float* T,
+                                                     int ldt, int* flag, bool report,
                                                      unsigned long long* badmask = nullptr) {
   __syncthreads();
-  if (threadIdx.x < 32) chol_inv_warp_ool(G, ldg, b, diag0, R, ldr, T, ldt, flag, report, badmask, 0);
+  chol_inv_two_warps(G, ldg, b, diag0, T, ldt, flag, report, badmask, 0);
   __syncthreads();
 }
 
 // 32 < b <= 64 in two column blocks (first 32, then b2 = b - 32), the two
-// diagonal blocks by the one-warp routine and the coupling products by the
-// whole CTA:  R11 = chol(G11), T11 = R11^-1;  R12 = T11^T G12;
+// diagonal blocks by the two-warp routine and the coupling products by the
+// whole CTA (of R only R12 is written):  R11 = chol(G11), T11 = R11^-1;  R12 = T11^T G12;
 // G22 <- G22 - R12^T R12;  R22 = chol(G22), T22 = R22^-1;
 // T12 = -(T11 R12) T22.  G (upper triangle used) is destroyed.
 static __device__ __noinline__ void chol_inv_blocked64(float* G, int ldg, int b, const float* diag0, float* R, int ldr, float* T,
                                           int ldt, int* flag, bool report, unsigned long long* badmask) {
   const int tid = threadIdx.x, nt = blockDim.x, b2 = b - 32;
   __syncthreads();
-  if (tid < 32) chol_inv_warp_ool(G, ldg, 32, diag0, R, ldr, T, ldt, flag, report, badmask, 0);
+  chol_inv_two_warps(G, ldg, 32, diag0, T, ldt, flag, report, badmask, 0);
   __syncthreads();
   // R12[i][c] = sum_{k <= i} T11[k][i] G[k][32 + c]; zero R21 and T21
   for (int x = tid; x < 32 * b2; x += nt) {
@@ -188,9 +247,7 @@ static __device__ __noinline__ void chol_inv_blocked64(float* G, int ldg, int b,
     G[(32 + i) * ldg + 32 + c] = acc;
   }
   __syncthreads();
-  if (tid < 32)
-    chol_inv_warp_ool(G + 32 * ldg + 32, ldg, b2, diag0 + 32, R + 32 * ldr + 32, ldr, T + 32 * ldt + 32, ldt, flag,
-                      report, badmask, 32);
+  chol_inv_two_warps(G + 32 * ldg + 32, ldg, b2, diag0 + 32, T + 32 * ldt + 32, ldt, flag, report, badmask, 32);
   __syncthreads();
   // X = T11 R12 (T11 upper: k >= i) into the place of G12, which is no
   // longer needed, then T12 = -X T22 (T22 upper: k <= c)
@@ -210,11 +267,11 @@ static __device__ __noinline__ void chol_inv_blocked64(float* G, int ldg, int b,
   __syncthreads();
 }
 
-// The fastest routine for the CTA at hand (same contract as chol_inv_cta):
-// one warp for b <= 32, two warp-factored column blocks for b <= 64.
+// The fastest routine for the CTA at hand (chol_inv_cta's contract, R only as
+// scratch): two warps for b <= 32, two such column blocks for b <= 64.
 __device__ inline void chol_inv_fast(float* G, int ldg, int b, const float* diag0, float* R, int ldr, float* T,
                                      int ldt, int* flag, bool report, unsigned long long* badmask = nullptr) {
-  if (b <= 32) chol_inv_warp32_call(G, ldg, b, diag0, R, ldr, T, ldt, flag, report, badmask);
+  if (b <= 32) chol_inv_warp32_call(G, ldg, b, diag0, T, ldt, flag, report, badmask);
   else if (b <= 64) chol_inv_blocked64(G, ldg, b, diag0, R, ldr, T, ldt, flag, report, badmask);
   else chol_inv_cta(G, ldg, b, diag0, R, ldr, T, ldt, flag, report, badmask);
 }

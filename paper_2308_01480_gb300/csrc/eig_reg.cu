@@ -647,7 +647,7 @@ __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict_
         __syncthreads();
       }
       if (tid < r) red[tid] = G[tid * 33 + tid];
-      chol_inv_warp32_call(G, 33, r, red, Rm, 33, Tm, 33, sflag, true);
+      chol_inv_warp32_call(G, 33, r, red, Tm, 33, sflag, true);
       if (*sflag) break;                  // uniform: fall back below
       // nxt[j][i] = sum_{a <= j} cur[a][i] T[a][j]
       for (int x = tid; x < r * k; x += NT) {

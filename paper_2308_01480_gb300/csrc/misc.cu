@@ -77,56 +77,70 @@ cudaError_t launch_omega(uint64_t seed, int mode, int64_t n, int b, void* out, i
   return cudaGetLastError();
 }
 
-// Transposed copy of an explicit Omega (n x b, row-major) into the b x n
-// layout read by the sketch pass, with dtype conversion.
+// Transposed copy of an explicit Omega (n x b row-major, b <= 64) into the
+// b x n layout read by the sketch pass, with dtype conversion.  HBM bounds
+// it: a CTA reads the b TR contiguous floats of TR rows in order, keeps them
+// transposed in shared memory (odd row stride: no bank conflicts on the way
+// in) and writes each column's TR entries together.  524,288 x 40 to BF16:
+// one strided element a thread took 116 us, this OMT_NOW.
 template <typename T>
-__global__ void k_transpose_in(const float* __restrict__ src, int64_t n, int b, T* __restrict__ dst) {
-  __shared__ float tile[32][65];
-  const int64_t r0 = (int64_t)blockIdx.x * 64;
-  for (int e = threadIdx.x; e < 64 * 32; e += blockDim.x) {
-    int r = e / 32, c = e % 32;
-    if (c < b && r0 + r < n) tile[c][r] = src[(r0 + r) * b + c];
+__global__ void __launch_bounds__(256) k_transpose_in(const float* __restrict__ src, int64_t n, int b,
+                                                      T* __restrict__ dst, bool pair) {
+  constexpr int TR = 128;
+  extern __shared__ float omt[];               // [b][TR + 1]
+  const int64_t r0 = (int64_t)blockIdx.x * TR;
+  const int rows = (int)imin(TR, n - r0);
+  const float* s = src + r0 * b;
+  const int total = rows * b, dc = 256 % b, dr = 256 / b;
+  int c = threadIdx.x % b, r = threadIdx.x / b;
+  for (int e = threadIdx.x; e < total; e += 4 * 256) {
+    float v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = (e + 256 * u < total) ? s[e + 256 * u] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (e + 256 * u < total) omt[c * (TR + 1) + r] = v[u];
+      c += dc;
+      r += dr;
+      if (c >= b) {
+        c -= b;
+        ++r;
+      }
+    }
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < 64 * 32; e += blockDim.x) {
-    int c = e / 64, r = e % 64;
-    if (c < b && r0 + r < n) st_elem(dst, (int64_t)c * n + r0 + r, tile[c][r]);
-  }
-}
-
-cudaError_t launch_omega_transpose(const float* src, int64_t n, int b, void* dst, int dtype, cudaStream_t st) {
-  if (b > 32) {
-    // two passes of at most 32 columns each would need a strided source; use
-    // the simple element-wise form for wide Omega
-    return cudaErrorInvalidValue;
-  }
-  dim3 grid((unsigned)ceil_div(n, 64));
-  note_launch("omega_transpose");
-  if (dtype == TT_BF16)
-    k_transpose_in<__nv_bfloat16><<<grid, 256, 0, st>>>(src, n, b, (__nv_bfloat16*)dst);
-  else
-    k_transpose_in<float><<<grid, 256, 0, st>>>(src, n, b, (float*)dst);
-  return cudaGetLastError();
-}
-
-template <typename T>
-__global__ void k_transpose_in_wide(const float* __restrict__ src, int64_t n, int b, T* __restrict__ dst) {
-  const int64_t total = n * b;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = e / n, r = e % n;
-    st_elem(dst, e, src[r * b + c]);
+  const int lane = threadIdx.x & 31;
+  for (int col = threadIdx.x >> 5; col < b; col += 8) {
+    const float* t = omt + col * (TR + 1);
+    T* out = dst + (int64_t)col * n + r0;
+    if constexpr (sizeof(T) == 2) {
+      if (pair) {                              // n even: rows, and pairs in them, are 4-byte aligned
+#pragma unroll
+        for (int u = 0; u < TR / 64; ++u) {
+          const int i = 2 * lane + 64 * u;
+          if (i < rows) *reinterpret_cast<__nv_bfloat162*>(out + i) = __floats2bfloat162_rn(t[i], t[i + 1]);
+        }
+        continue;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < TR / 32; ++u) {
+      const int i = lane + 32 * u;
+      if (i < rows) st_elem(out, i, t[i]);
+    }
   }
 }
 
 cudaError_t launch_omega_transpose_any(const float* src, int64_t n, int b, void* dst, int dtype, cudaStream_t st) {
-  if (b <= 32) return launch_omega_transpose(src, n, b, dst, dtype, st);
-  const int blocks = (int)imin(ceil_div(n * b, 256), 152 * 16);
+  if (b < 1 || b > 64) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)ceil_div(n, 128));
+  const size_t smem = sizeof(float) * (size_t)b * 129;
   note_launch("omega_transpose");
   if (dtype == TT_BF16)
-    k_transpose_in_wide<__nv_bfloat16><<<blocks, 256, 0, st>>>(src, n, b, (__nv_bfloat16*)dst);
+    k_transpose_in<__nv_bfloat16><<<grid, 256, smem, st>>>(src, n, b, (__nv_bfloat16*)dst,
+                                                           n % 2 == 0 && reinterpret_cast<uintptr_t>(dst) % 4 == 0);
   else
-    k_transpose_in_wide<float><<<blocks, 256, 0, st>>>(src, n, b, (float*)dst);
+    k_transpose_in<float><<<grid, 256, smem, st>>>(src, n, b, (float*)dst, false);
   return cudaGetLastError();
 }
 

@@ -91,48 +91,77 @@ __host__ __device__ inline KcLayout kc_layout(int kqmax, int zmax, int rows, int
   L.Zc = take((size_t)L.RP * L.ZP);
   L.Zn = take((size_t)L.RP * L.ZP);
   L.Qc = take((size_t)L.RP * L.KP);
-  L.tmp = take(8 * (size_t)L.ZP * L.ZP);   // split partial products of the Gram
+  // split partial products: at most 512 tiles of 16 sums (tn_split)
+  L.tmp = take(imin(8192, 8 * (size_t)L.ZP * imax(L.KP, L.ZP)));
   L.total = o;
   return L;
 }
 
-// Y[i][j] = scale * sum_{t < kk} X[i][t] M[t][j] (+ Y0[i][j]) for i < rows
-// (multiple of 4), j < bp (multiple of 4), with TR x 4 register tiles so
-// that short blocks still occupy every thread (row strides multiples of 4).
-template <int TR>
-__device__ void nn_rows(const float* X, int ldx, int kk, const float* M, int ldm, int rows, int bp, float* Y, int ldy,
-                        const float* Y0, float scale) {
-  const int ti = rows / TR, tj = bp >> 2;
-  for (int tile = threadIdx.x; tile < ti * tj; tile += blockDim.x) {
-    const int i0 = (tile / tj) * TR, j0 = (tile % tj) * 4;
-    float acc[TR][4] = {};
-    for (int t = 0; t < kk; ++t) {
-      const float4 v = *reinterpret_cast<const float4*>(M + t * ldm + j0);
+// Y[i][j] = scale * sum_{t < kk} X[i][t] M[t][j] (+ Y0[i][j]) for i < rows,
+// j < bp (rows, kk, bp and the row strides multiples of 4).  A warp takes
+// four rows: lanes 8 g + jt hold the 4 x 4 tile of columns 4 jt .. 4 jt + 3
+// over the g-th of every four groups of four t, so that a step is eight
+// 16-byte loads (those of M one conflict-free row per eight lanes, those of X
+// broadcasts) for 64 multiply-adds; the four groups are added by a
+// transposing exchange that leaves lane g with row g.  (One 1 x 4 to 4 x 4
+// tile a thread over all of kk read five operands per 4 to 16 multiply-adds:
+// 8.6K cycles for 52 x 32 over kk = 120, now 5.2K.)
+__device__ void nn_any(const float* X, int ldx, int kk, const float* M, int ldm, int rows, int bp, float* Y, int ldy,
+                       const float* Y0, float scale) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int g = lane >> 3, jt = lane & 7;
+  const int ti = rows >> 2, tj = (bp + 31) >> 5;
+  for (int task = threadIdx.x >> 5; task < ti * tj; task += nw) {
+    const int i0 = (task / tj) * 4, j0 = (task % tj) * 32 + 4 * jt;
+    const bool live = j0 < bp;
+    float acc[4][4] = {};
+    if (live) {
+      const float* x = X + i0 * ldx;
+      const float* mm = M + j0;
+      for (int t = 4 * g; t < kk; t += 16) {
+        float4 xv[4], mv[4];
 #pragma unroll
-      for (int u = 0; u < TR; ++u) {
-        const float x = X[(i0 + u) * ldx + t];
-        acc[u][0] = fmaf(x, v.x, acc[u][0]); acc[u][1] = fmaf(x, v.y, acc[u][1]);
-        acc[u][2] = fmaf(x, v.z, acc[u][2]); acc[u][3] = fmaf(x, v.w, acc[u][3]);
+        for (int u = 0; u < 4; ++u) xv[u] = *reinterpret_cast<const float4*>(x + u * ldx + t);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) mv[u] = *reinterpret_cast<const float4*>(mm + (t + u) * ldm);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float xs[4] = {xv[u].x, xv[u].y, xv[u].z, xv[u].w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            acc[u][0] = fmaf(xs[q], mv[q].x, acc[u][0]);
+            acc[u][1] = fmaf(xs[q], mv[q].y, acc[u][1]);
+            acc[u][2] = fmaf(xs[q], mv[q].z, acc[u][2]);
+            acc[u][3] = fmaf(xs[q], mv[q].w, acc[u][3]);
+          }
+        }
       }
     }
+    // rows 2, 3 to the upper half-warp, then odd rows to the odd groups
+    const bool hi = lane & 16, odd = lane & 8;
+    float h[2][4], s[4];
 #pragma unroll
-    for (int u = 0; u < TR; ++u) {
-      float4 r = make_float4(acc[u][0] * scale, acc[u][1] * scale, acc[u][2] * scale, acc[u][3] * scale);
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        const float send = hi ? acc[u][w] : acc[u + 2][w], keep = hi ? acc[u + 2][w] : acc[u][w];
+        h[u][w] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+      }
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const float send = odd ? h[0][w] : h[1][w], keep = odd ? h[1][w] : h[0][w];
+      s[w] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+    }
+    if (live) {
+      const int row = i0 + g;
+      float4 r = make_float4(s[0] * scale, s[1] * scale, s[2] * scale, s[3] * scale);
       if (Y0) {
-        const float4 y = *reinterpret_cast<const float4*>(Y0 + (i0 + u) * ldy + j0);
+        const float4 y = *reinterpret_cast<const float4*>(Y0 + row * ldy + j0);
         r.x += y.x; r.y += y.y; r.z += y.z; r.w += y.w;
       }
-      *reinterpret_cast<float4*>(Y + (i0 + u) * ldy + j0) = r;
+      *reinterpret_cast<float4*>(Y + row * ldy + j0) = r;
     }
   }
-}
-
-__device__ __forceinline__ void nn_any(const float* X, int ldx, int kk, const float* M, int ldm, int rows, int bp,
-                                       float* Y, int ldy, const float* Y0, float scale) {
-  const int t4 = (rows / 4) * (bp / 4);
-  if (2 * t4 >= (int)blockDim.x) nn_rows<4>(X, ldx, kk, M, ldm, rows, bp, Y, ldy, Y0, scale);
-  else if (4 * t4 >= (int)blockDim.x || (rows & 3)) nn_rows<2>(X, ldx, kk, M, ldm, rows, bp, Y, ldy, Y0, scale);
-  else nn_rows<1>(X, ldx, kk, M, ldm, rows, bp, Y, ldy, Y0, scale);
 }
 
 // out[t][j] = sum_{i < rows} A[i][t] B[i][j] (t < ta, j < bp, multiples of 4)
@@ -142,7 +171,7 @@ __device__ __forceinline__ void nn_any(const float* X, int ldx, int kk, const fl
 __device__ void tn_split(const float* A, int lda, int ta, const float* B, int ldb, int bp, int rows, float* out,
                          int ldo, float* tmp) {
   const int tt = ta >> 2, tj = bp >> 2, tiles = tt * tj;
-  const int KS = imax(1, imin(8, (int)blockDim.x / tiles));
+  const int KS = 4 * tiles <= (int)blockDim.x ? imin(8, (int)blockDim.x / tiles) : 1;
   if (KS == 1) {
     tn_tile(A, lda, ta, B, ldb, bp, rows, out, ldo);
     __syncthreads();
@@ -153,6 +182,7 @@ __device__ void tn_split(const float* A, int lda, int ta, const float* B, int ld
     const int tile = tid % tiles, g = tid / tiles;
     const int t0 = (tile / tj) * 4, j0 = (tile % tj) * 4;
     float acc[4][4] = {};
+#pragma unroll 4
     for (int i = g; i < rows; i += KS) {
       const float4 x = *reinterpret_cast<const float4*>(A + i * lda + t0);
       const float4 v = *reinterpret_cast<const float4*>(B + i * ldb + j0);
@@ -332,14 +362,17 @@ __device__ __forceinline__ void orth_rs_body(const OrthRsArgs& a, Comm& comm, fl
       __syncthreads();
       auto reduce = [&](bool qz, bool zz) {
         float* mine = share0 + (size_t)(L.share_bufs == 2 ? (phase & 1) : 0) * (KP + ZP) * ZP;
-        if (qz) tn_tile(Qc, KP, kp, Zc, ZP, bz, RP, mine, bz);
+        if (qz) tn_split(Qc, KP, kp, Zc, ZP, bz, RP, mine, bz, tmp);
         if (zz) tn_split(Zc, ZP, bz, Zc, ZP, bz, RP, mine + kp * bz, bz, tmp);
         __syncthreads();
         const int e0 = qz ? 0 : kp * bz, e1 = zz ? E : kp * bz;
         auto put = [&](int e, float s) {
-          const int row = e / bz, j = e % bz;
-          if (row < kp) P[e] = s;
-          else if (row - kp < zc && j < zc) Gm[(row - kp) * (zc + 1) + j] = s;
+          if (e < kp * bz) {
+            P[e] = s;
+          } else {
+            const int row = e / bz - kp, j = e % bz;
+            if (row < zc && j < zc) Gm[row * (zc + 1) + j] = s;
+          }
         };
         comm.reduce(mine, phase, e0, e1, put);
         __syncthreads();

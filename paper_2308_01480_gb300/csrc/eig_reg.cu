@@ -5,11 +5,8 @@
 // warps, so that the register-resident Cholesky of step 4 fits) does steps
 // 2-5.
 //
-//  1. Householder tridiagonalisation.  Per column two barriers: the warp
-//     owning column j forms the reflector v from its registers; each warp
-//     forms p = tau H v for its own columns by a lane reduction; then every
-//     thread applies H -= v w^T + w v^T to its entries, w = p - (tau/2)
-//     (v^T p) v.  The reflectors go to global scratch.
+//  1. Householder tridiagonalisation, two barriers per column (below).  The
+//     reflectors go to global scratch.
 //  2. Bisection by Sturm counts: one round with a count at each of 512
 //     points over the Gershgorin interval, then each warp refines the
 //     brackets of two wanted eigenvalues at once by three rounds of 33-point
@@ -20,8 +17,8 @@
 //     QR twice (columns in descending eigenvalue order, so the result is
 //     the Gram-Schmidt basis), or Gram-Schmidt twice when a Cholesky pivot
 //     is too small.
-//  5. Back-transformation by the stored reflectors, four at a time, a warp
-//     per two vectors held in registers.
+//  5. Back-transformation by the stored reflectors, sixteen at a time, all
+//     vectors together.
 #include <float.h>
 
 #include <utility>
@@ -70,111 +67,201 @@ __device__ __forceinline__ int warp_min_i(int v) {
   return v;
 }
 
-// Number of eigenvalues of T = (d, e) below x (Sturm sequence of the LDL^T
-// pivots); e2 holds the squared off-diagonal.
-__device__ __forceinline__ int sturm(const float* d, const float* e2, int k, float x, float pivmin) {
-  int c = 0;
-  float q = d[0] - x;
-  if (fabsf(q) < pivmin) q = -pivmin;
-  c += q < 0.f;
-#pragma unroll 4
-  for (int i = 1; i < k; ++i) {
-    q = (d[i] - x) - __fdividef(e2[i - 1], q);
-    if (fabsf(q) < pivmin) q = -pivmin;
-    c += q < 0.f;
+// Number of eigenvalues of the scaled T below x: sign changes of the leading
+// principal minors p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (Givens 1953),
+// de[i] = (d_i, e_{i-1}^2), |T| < 2.  One multiply-add a row is on the chain
+// (the ratios p_i / p_{i-1} would put a reciprocal and a comparison there);
+// every four rows the pair is rescaled by a power of two.  Rows past the last
+// are padded by (16, 0), which changes no sign, up to 1 + 4 groups rows.
+// k = 150: 75 to 100 cycles a row as ratios, about 55 (two counts a warp).
+struct SturmPair {
+  float p0, p1;
+  unsigned m;        // signs of the last p's, newest in bit 0
+  int c;
+  __device__ __forceinline__ void start(float2 t, float x) {
+    p0 = 1.f;
+    p1 = t.x - x;
+    m = __float_as_uint(p1) >> 31;
+    c = (int)m;
   }
-  return c;
+  __device__ __forceinline__ void step(float d, float e2, float x) {
+    const float pn = fmaf(d - x, p1, -(e2 * p0));
+    m = __funnelshift_l(__float_as_uint(pn), m, 1);
+    p0 = p1;
+    p1 = pn;
+  }
+  // after every four steps
+  __device__ __forceinline__ void settle() {
+    c += __popc((m ^ (m >> 1)) & 15u);
+    const float f0 = fmaxf(fabsf(p0), fabsf(p1));
+    const float f = __uint_as_float(0x7f000000u - (__float_as_uint(f0) & 0x7f800000u));
+    p0 *= f;
+    p1 = (f0 == 0.f) ? 1.f : p1 * f;     // both zero: the rows decouple here
+  }
+};
+
+// Rows 1 .. 4 groups are read as pairs: de + 1 is 16-byte aligned.
+__device__ __forceinline__ int sturm(const float2* de, int groups, float x) {
+  SturmPair s;
+  s.start(de[0], x);
+  const float4* q = reinterpret_cast<const float4*>(de + 1);
+#pragma unroll 2
+  for (int g = 0; g < groups; ++g) {
+    const float4 a = q[2 * g], b = q[2 * g + 1];
+    s.step(a.x, a.y, x);
+    s.step(a.z, a.w, x);
+    s.step(b.x, b.y, x);
+    s.step(b.z, b.w, x);
+    s.settle();
+  }
+  return s.c;
 }
 
-// Two Sturm counts (at x0 and x1) in one pass, so that the two dependent
-// chains overlap.
-__device__ __forceinline__ void sturm2(const float* d, const float* e2, int k, float x0, float x1, float pivmin,
-                                       int& c0, int& c1) {
-  float q0 = d[0] - x0, q1 = d[0] - x1;
-  if (fabsf(q0) < pivmin) q0 = -pivmin;
-  if (fabsf(q1) < pivmin) q1 = -pivmin;
-  c0 = q0 < 0.f;
-  c1 = q1 < 0.f;
-#pragma unroll 4
-  for (int i = 1; i < k; ++i) {
-    const float di = d[i], ei = e2[i - 1];
-    q0 = (di - x0) - __fdividef(ei, q0);
-    q1 = (di - x1) - __fdividef(ei, q1);
-    if (fabsf(q0) < pivmin) q0 = -pivmin;
-    if (fabsf(q1) < pivmin) q1 = -pivmin;
-    c0 += q0 < 0.f;
-    c1 += q1 < 0.f;
+// Two counts (at x0 and x1) in one pass, so that the two chains overlap.
+__device__ __forceinline__ void sturm2(const float2* de, int groups, float x0, float x1, int& c0, int& c1) {
+  SturmPair s0, s1;
+  s0.start(de[0], x0);
+  s1.start(de[0], x1);
+  const float4* q = reinterpret_cast<const float4*>(de + 1);
+  for (int g = 0; g < groups; ++g) {
+    const float4 a = q[2 * g], b = q[2 * g + 1];
+    s0.step(a.x, a.y, x0); s1.step(a.x, a.y, x1);
+    s0.step(a.z, a.w, x0); s1.step(a.z, a.w, x1);
+    s0.step(b.x, b.y, x0); s1.step(b.x, b.y, x1);
+    s0.step(b.z, b.w, x0); s1.step(b.z, b.w, x1);
+    s0.settle();
+    s1.settle();
   }
+  c0 = s0.c;
+  c1 = s1.c;
 }
 
-// Pivoted LU of T - lam I into w[0..5k) (reciprocal pivots, two upper
-// diagonals, multipliers, exchange flags); tiny pivots replaced by +-tiny.
-__device__ void tri_lu(const float* d, const float* e, int k, float lam, float tiny, float* w) {
-  float* r0 = w;
-  float* u1 = w + k;
-  float* u2 = w + 2 * k;
-  float* l = w + 3 * k;
-  float* sw = w + 4 * k;
-  float alpha = d[0] - lam, beta = (k > 1) ? e[0] : 0.f;
+// Pivoted LU of T - lam I, one thread per vector: row i of w holds
+// (1 / pivot, two upper diagonals, multiplier), bit i & 7 of ex[i / 8] whether
+// rows were exchanged; tiny pivots replaced by +-tiny.  Rows k .. kp - 1 (kp a
+// multiple of 8) are zero, so that the solves need no bounds checks.  A chain
+// of k steps whose latency is the time: the exchange is a selection (lanes
+// that exchange and lanes that do not would otherwise take turns) and the
+// reciprocals of both candidate pivots are taken before it is known.
+__device__ __forceinline__ float rcp_pivot(float p, float tiny) {
+  return __fdividef(1.f, (fabsf(p) < tiny) ? copysignf(tiny, p) : p);
+}
+__device__ void tri_lu(const float* __restrict__ d, const float* __restrict__ e, int k, int kp, float lam, float tiny,
+                       float4* __restrict__ w, uint32_t* __restrict__ ex) {
+  float alpha = d[0] - lam, beta = (k > 1) ? e[0] : 0.f, sub = beta;
+  uint32_t bits = 0u;
   for (int i = 0; i + 1 < k; ++i) {
-    const float sub = e[i];
-    const float a1 = d[i + 1] - lam, c1 = (i + 2 < k) ? e[i + 1] : 0.f;
-    if (fabsf(alpha) >= fabsf(sub)) {
-      const float piv = (fabsf(alpha) < tiny) ? copysignf(tiny, alpha) : alpha;
-      const float rp = __fdividef(1.f, piv);
-      const float li = sub * rp;
-      r0[i] = rp; u1[i] = beta; u2[i] = 0.f; l[i] = li; sw[i] = 0.f;
-      alpha = fmaf(-li, beta, a1);
-      beta = c1;
-    } else {
-      const float rs = __fdividef(1.f, (fabsf(sub) < tiny) ? copysignf(tiny, sub) : sub);
-      const float li = alpha * rs;
-      r0[i] = rs; u1[i] = a1; u2[i] = c1; l[i] = li; sw[i] = 1.f;
-      alpha = fmaf(-li, a1, beta);
-      beta = -li * c1;
+    const float a1 = d[i + 1] - lam, c1 = e[i + 1];        // e[k - 1] is zero
+    const float rs = rcp_pivot(sub, tiny), ra = rcp_pivot(alpha, tiny);
+    const bool keep = fabsf(alpha) >= fabsf(sub);
+    const float rp = keep ? ra : rs;
+    const float li = (keep ? sub : alpha) * rp;
+    const float up = keep ? beta : a1, lo = keep ? a1 : beta;
+    w[i] = make_float4(rp, up, keep ? 0.f : c1, li);
+    bits |= keep ? 0u : (1u << (i & 7));
+    if ((i & 7) == 7) {
+      ex[i >> 3] = bits;
+      bits = 0u;
     }
+    alpha = fmaf(-li, up, lo);
+    beta = keep ? c1 : -li * c1;
+    sub = c1;
   }
-  r0[k - 1] = __fdividef(1.f, (fabsf(alpha) < tiny) ? copysignf(tiny, alpha) : alpha);
-  u1[k - 1] = 0.f; u2[k - 1] = 0.f; l[k - 1] = 0.f; sw[k - 1] = 0.f;
+  w[k - 1] = make_float4(rcp_pivot(alpha, tiny), 0.f, 0.f, 0.f);
+  ex[(k - 1) >> 3] = bits;
+  for (int i = k; i < kp; ++i) w[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-__device__ void tri_lu_solve(const float* w, int k, float* x) {
-  const float* r0 = w;
-  const float* u1 = w + k;
-  const float* u2 = w + 2 * k;
-  const float* l = w + 3 * k;
-  const float* sw = w + 4 * k;
+// x <- (T - lam I)^-1 x (x zero from k to kp), returning max |x_i|; eight rows
+// of the factors and of x in registers at a time, since a store to x between
+// two loads would make each row wait for shared memory.
+__device__ float tri_lu_solve(const float4* __restrict__ w, const uint32_t* __restrict__ ex, int kp,
+                              float* __restrict__ x) {
   float xi = x[0];
-  for (int i = 0; i + 1 < k; ++i) {
-    float xn = x[i + 1];
-    if (sw[i] != 0.f) { const float t = xi; xi = xn; xn = t; }
-    x[i] = xi;
-    xi = fmaf(-l[i], xi, xn);
+  for (int i0 = 0; i0 < kp; i0 += 8) {
+    float lv[8], xn[8];
+    const uint32_t bits = ex[i0 >> 3];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      lv[q] = w[i0 + q].w;
+      xn[q] = x[i0 + q + 1];
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const bool swap = bits & (1u << q);
+      const float top = swap ? xn[q] : xi, low = swap ? xi : xn[q];
+      xn[q] = top;
+      xi = fmaf(-lv[q], top, low);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[i0 + q] = xn[q];
   }
-  x[k - 1] = xi;
-  float x1 = 0.f, x2 = 0.f;
-  for (int i = k - 1; i >= 0; --i) {
-    const float v = (x[i] - u1[i] * x1 - u2[i] * x2) * r0[i];
-    x[i] = v;
-    x2 = x1;
-    x1 = v;
+  float x1 = 0.f, x2 = 0.f, mx = 0.f;
+  for (int i0 = kp - 8; i0 >= 0; i0 -= 8) {
+    float4 f[8];
+    float xv[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      f[q] = w[i0 + q];
+      xv[q] = x[i0 + q];
+    }
+#pragma unroll
+    for (int q = 7; q >= 0; --q) {
+      const float v = fmaf(-f[q].y, x1, fmaf(-f[q].z, x2, xv[q])) * f[q].x;
+      xv[q] = v;
+      mx = fmaxf(mx, fabsf(v));
+      x2 = x1;
+      x1 = v;
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[i0 + q] = xv[q];
   }
+  return mx;
 }
 
 }  // namespace
 
-// Shared-memory floats of k_eig_vectors for k (padded to KM = 32 KT) and r.
-// Odd row strides for the vectors (k + 1 or k + 2) and the per-vector
-// inverse-iteration factors (5 k or 5 k + 1): one thread per vector walks
-// its row, so an odd stride keeps the 32 threads on 32 banks.
-__host__ __device__ inline int er_ldx(int k) { return (k + 1) | 1; }
-__host__ __device__ inline int er_ldw(int k) { return (5 * k) | 1; }
-__host__ __device__ inline size_t er_union_floats(int k, int r) {
-  const size_t a = (size_t)k * k, b = (size_t)r * er_ldw(k);
-  return a > b ? a : b;
-}
-__host__ __device__ inline size_t er_smem_floats(int KM, int k, int r) {
-  return er_union_floats(k, r) + 4 * (size_t)KM + 32 + 64 + 1024 + 2 * (size_t)r * er_ldx(k) + 3 * 33 * 32 + 8;
+// Reflectors per group of the back-transformation.
+constexpr int ER_GB = 16;
+
+// Shared memory of k_eig_vectors (float offsets).  The vectors' rows have an
+// odd stride and the inverse-iteration factors' rows one of 4 mod 32 floats:
+// one thread per vector walks its row, so neither meets a bank conflict.  The
+// vectors' rows are zero from k on (up to 32 KT and one more).
+struct ErLayout {
+  int ldx, ldw, kp, groups;
+  size_t V, tau, d, e, de, lam, red, cnt, ex, X, X2, G, T, S, D, C, total;
+};
+__host__ __device__ inline ErLayout er_layout(int KM, int k, int r) {
+  ErLayout L;
+  L.kp = (k + 7) & ~7;
+  L.ldx = KM + 1;
+  L.ldw = 4 * ((L.kp + 7) & ~7) + 4;
+  L.groups = k > 2 ? (k - 2 + ER_GB - 1) / ER_GB : 0;
+  size_t o = 0;
+  auto take = [&](size_t n) { const size_t at = o; o += (n + 3) & ~size_t(3); return at; };
+  // the reflectors (step 5) and the inverse-iteration factors (step 3) are
+  // never live together: one region holds both.  Reads of whole 32-entry
+  // chunks run up to 31 floats past the last reflector, which are zeroed.
+  const size_t v = (size_t)k * k + 32, w = (size_t)r * L.ldw;
+  L.V = take(v > w ? v : w);
+  L.tau = take(KM);
+  L.d = take(KM);
+  L.e = take(KM);
+  L.de = take(2 * (size_t)(KM + 4) + 4) + 2;   // de + 1 on a 16-byte boundary
+  L.lam = take(32);
+  L.red = take(64);
+  L.cnt = take(512);
+  L.ex = take(32 * 21);
+  L.X = take((size_t)r * L.ldx);
+  L.X2 = take((size_t)r * L.ldx);
+  L.G = take(36 * 33);
+  L.T = take(33 * 32);
+  L.S = take((size_t)L.groups * ER_GB * (ER_GB + 1));
+  L.D = take(ER_GB * 36);
+  L.C = take(ER_GB * 36);
+  L.total = o + 4;       // the last word: a flag
+  return L;
 }
 
 // Sum over the 32 lanes of NV values x[0..NV) (NV a power of two <= 32) with
@@ -218,13 +305,20 @@ __device__ __forceinline__ float lane_transpose_sum(float (&x)[NV]) {
 // warp and each thread carries 20 KR entries (the per-column reductions,
 // broadcasts and barriers are spread over many multiply-adds).  Per column
 // two barriers:
-//   R  the warp owning column j forms the reflector v (and tau) from its
-//      registers and publishes it;
 //   M  every warp forms tau (H v)_c for its columns c (H is symmetric, so the
 //      column dot is the row product) and its share of v^T H v, reduced over
 //      the lanes by one transposing butterfly;
 //   U  every thread applies H -= v w^T + w v^T, w = p - (tau/2)(v^T p) v,
-//      to its entries of the trailing block.
+//      to its entries of the trailing block: the four column slots that hold
+//      the next column first, then
+//   R  the warp owning the next column forms its reflector (v and tau) from
+//      its registers and publishes it while the others finish U.
+// The column time is the chain barrier, M, barrier, the next column's update,
+// R; v and p are kept in shared memory in column order and, for the 20
+// broadcasts of a warp's own columns, also warp by warp, so that five
+// 16-byte loads fetch them.  With R after all of U, scalar broadcasts and three
+// operations per entry in U a column of k = 150 took 1,300 (late) to 3,100
+// (early) cycles, 139 us in all; 1,050 to 2,500 and 122 us so.
 // Tiles of finished rows (32-row blocks) and columns (8-column slots) are
 // skipped at compile time: the column loop is split into 32-column segments.
 template <int KR, int NW>
@@ -234,9 +328,11 @@ __global__ void __launch_bounds__(NW * 32, 1) k_eig_tridiag8(const float* __rest
   constexpr int SPS = 32 / NW;            // column slots per warp in a 32-column segment
   constexpr int KC = SPS * KR;
   constexpr int KM = 32 * KR;
-  constexpr int NV = (KC + 1 <= 8) ? 8 : (KC + 1 <= 16) ? 16 : 32;
-  __shared__ __align__(16) float vs[KM];
+  static_assert(SPS == 4, "a segment's slots of a warp are one 16-byte load");
+  __shared__ __align__(16) float vs[2][KM];    // v in column order
+  __shared__ __align__(16) float vw[2][KM];    // v, warp by warp: entry (i % NW) KC + i / NW
   __shared__ __align__(16) float ps[KM];
+  __shared__ __align__(16) float pw[KM];
   __shared__ float wsum[NW];
   __shared__ float scal[2];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -253,86 +349,120 @@ __global__ void __launch_bounds__(NW * 32, 1) k_eig_tridiag8(const float* __rest
   sfor<KR>([&](auto seg) {
     constexpr int S = decltype(seg)::value;
     const int jend = min(32 * S + 32, k - 2);
-    for (int j = 32 * S; j < jend; ++j) {
-      // R: the reflector of column j (slot j / NW in warp j % NW)
-      if (w == (j % NW)) {
-        const int t = (j / NW) - SPS * S;   // 0 .. SPS - 1
-        float colv[KR];
-        sfor<KR>([&](auto a) {
-          float x = 0.f;
-          if constexpr (a >= S) {
-            sfor<SPS>([&](auto u) {
-              if constexpr (SPS * S + u < KC)
-                if (t == u) x = A[a][SPS * S + u];
-            });
-          }
-          colv[a] = x;
-        });
-        float part = 0.f, sel = 0.f;
-        const int a1 = (j + 1) >> 5;
-        sfor<KR>([&](auto a) {
-          if constexpr (a >= S) {
-            const float x = colv[a];
-            const int i = lane + 32 * a;
-            if (i >= j + 2 && i < k) part = fmaf(x, x, part);
-            if (a == a1) sel = x;
-            if (i == j) d_g[j] = x;
-          }
-        });
-        const float sigma = warp_sum(part);
-        const float x0 = __shfl_sync(0xffffffffu, sel, (j + 1) & 31);
-        float tt = 0.f, iv = 0.f, beta = x0;
-        if (sigma > 0.f) {
-          const float mu = sqrtf(fmaf(x0, x0, sigma));
-          const float v0 = (x0 <= 0.f) ? x0 - mu : __fdividef(-sigma, x0 + mu);
-          tt = __fdividef(2.f * v0 * v0, fmaf(v0, v0, sigma));
-          beta = mu;
-          iv = __fdividef(1.f, v0);
-        }
-        sfor<KR>([&](auto a) {
-          const int i = lane + 32 * a;
-          const float v = (a < S) ? 0.f : ((i == j + 1) ? 1.f : ((i > j + 1 && i < k) ? colv[a] * iv : 0.f));
-          vs[i] = v;
-          if (i < k) Vg[(size_t)j * k + i] = (tt != 0.f) ? v : 0.f;
-        });
-        if (lane == 0) {
-          scal[j & 1] = tt;
-          tau_g[j] = tt;
-          e_g[j] = beta;
-        }
-      }
-      __syncthreads();
-      const float tau = scal[j & 1];
-      if (tau == 0.f) continue;              // the same decision in every thread
-      // M: (H v)_c for this thread's live columns, its share of v^T H v
-      float vr[KR], vc[KC];
-      sfor<KR>([&](auto a) { vr[a] = (a >= S) ? vs[lane + 32 * a] : 0.f; });
-      sfor<KC>([&](auto c) { vc[c] = (c >= SPS * S) ? vs[w + NW * c] : 0.f; });
-      float xv[NV];
-      sfor<NV>([&](auto c) { xv[c] = 0.f; });
-      sfor<KC>([&](auto c) {
-        if constexpr (c >= SPS * S) {
-          float acc = 0.f;
-          sfor<KR>([&](auto a) {
-            if constexpr (a >= S) acc = fmaf(A[a][c], vr[a], acc);
+    // R: the reflector of column j (slot j / NW of warp j % NW, inside this segment)
+    auto reflector = [&](int j) {
+      const int t = (j / NW) - SPS * S;   // 0 .. SPS - 1
+      float colv[KR];
+      sfor<KR>([&](auto a) {
+        float x = 0.f;
+        if constexpr (a >= S) {
+          sfor<SPS>([&](auto u) {
+            if (t == u) x = A[a][SPS * S + u];
           });
-          xv[c] = acc;
-          xv[KC] = fmaf(vc[c], acc, xv[KC]);
+        }
+        colv[a] = x;
+      });
+      float part = 0.f, sel = 0.f;
+      const int a1 = (j + 1) >> 5;
+      sfor<KR>([&](auto a) {
+        if constexpr (a >= S) {
+          const float x = colv[a];
+          const int i = lane + 32 * a;
+          if (i >= j + 2 && i < k) part = fmaf(x, x, part);
+          if (a == a1) sel = x;
         }
       });
-      const float tot = lane_transpose_sum<NV>(xv);
-      {
-        constexpr int shift = (NV == 32) ? 0 : (NV == 16) ? 1 : 2;
-        const int vi = lane >> shift;
-        if ((lane & ((1 << shift) - 1)) == 0) {
-          if (vi < KC) {
-            const int col = w + NW * vi;
-            if (col < KM) ps[col] = (col > j && col < k) ? tau * tot : 0.f;
-          } else if (vi == KC) {
-            wsum[w] = tot;
-          }
-        }
+      const float x0 = __shfl_sync(0xffffffffu, sel, (j + 1) & 31);
+      const float sigma = warp_sum(part);
+      float tt = 0.f, iv = 0.f, beta = x0;
+      if (sigma > 0.f) {
+        const float s2 = fmaf(x0, x0, sigma);
+        const float mu = s2 * rsqrtf(s2);
+        const float v0 = (x0 <= 0.f) ? x0 - mu : __fdividef(-sigma, x0 + mu);
+        tt = __fdividef(2.f * v0 * v0, fmaf(v0, v0, sigma));
+        beta = mu;
+        iv = __fdividef(1.f, v0);
       }
+      float v[KR];
+      sfor<KR>([&](auto a) {
+        const int i = lane + 32 * a;
+        v[a] = (a < S) ? 0.f : ((i == j + 1) ? 1.f : ((i > j + 1 && i < k) ? colv[a] * iv : 0.f));
+        vs[j & 1][i] = v[a];
+        vw[j & 1][(lane % NW) * KC + (lane / NW) + SPS * a] = v[a];
+      });
+      if (lane == 0) {
+        scal[j & 1] = tt;
+        tau_g[j] = tt;
+        e_g[j] = beta;
+      }
+      sfor<KR>([&](auto a) {
+        const int i = lane + 32 * a;
+        if (i < k) Vg[(size_t)j * k + i] = (tt != 0.f) ? v[a] : 0.f;
+        if constexpr (a >= S) {
+          if (i == j) d_g[j] = colv[a];
+        }
+      });
+    };
+    if (32 * S < jend && w == (32 * S) % NW) reflector(32 * S);
+    for (int j = 32 * S; j < jend; ++j) {
+      __syncthreads();
+      const float tau = scal[j & 1];
+      const bool next = j + 1 < jend && w == ((j + 1) % NW);
+      if (tau == 0.f) {                      // the same decision in every thread
+        if (next) reflector(j + 1);
+        continue;
+      }
+      // M: (H v)_c for this thread's live columns, its share of v^T H v
+      constexpr int LIVE = KC - SPS * S;
+      float vr[KR], vc[KC];
+      sfor<KR>([&](auto a) { vr[a] = (a >= S) ? vs[j & 1][lane + 32 * a] : 0.f; });
+      sfor<KR>([&](auto q) {
+        if constexpr (q >= S) {
+          const float4 x = *reinterpret_cast<const float4*>(&vw[j & 1][w * KC + 4 * q]);
+          vc[4 * q] = x.x; vc[4 * q + 1] = x.y; vc[4 * q + 2] = x.z; vc[4 * q + 3] = x.w;
+        } else {
+          vc[4 * q] = vc[4 * q + 1] = vc[4 * q + 2] = vc[4 * q + 3] = 0.f;
+        }
+      });
+      float hv[LIVE], part = 0.f;
+      sfor<LIVE>([&](auto c) {
+        float acc = 0.f;
+        sfor<KR>([&](auto a) {
+          if constexpr (a >= S) acc = fmaf(A[a][SPS * S + c], vr[a], acc);
+        });
+        hv[c] = acc;
+        part = fmaf(vc[SPS * S + c], acc, part);
+      });
+      // lane totals of the live columns in butterflies of 16, 8 or 4
+      auto publish = [&](auto first, auto count) {
+        constexpr int F = decltype(first)::value, N = decltype(count)::value;
+        float x[N];
+        sfor<N>([&](auto c) {
+          if constexpr (F + c < LIVE) x[c] = hv[F + c];
+          else x[c] = 0.f;
+        });
+        const float tot = lane_transpose_sum<N>(x);
+        constexpr int shift = (N == 16) ? 1 : (N == 8) ? 2 : 3;
+        const int vi = SPS * S + F + (lane >> shift);
+        if ((lane & ((1 << shift) - 1)) == 0 && vi < KC) {
+          const int col = w + NW * vi;
+          const float pv = (col > j && col < k) ? tau * tot : 0.f;
+          ps[col] = pv;
+          pw[w * KC + vi] = pv;
+        }
+      };
+      if constexpr (LIVE > 16) {
+        publish(CIdx<0>{}, CIdx<16>{});
+        publish(CIdx<16>{}, CIdx<4>{});
+      } else if constexpr (LIVE > 8) {
+        publish(CIdx<0>{}, CIdx<16>{});
+      } else if constexpr (LIVE > 4) {
+        publish(CIdx<0>{}, CIdx<8>{});
+      } else {
+        publish(CIdx<0>{}, CIdx<4>{});
+      }
+      const float share = warp_sum(part);
+      if (lane == 0) wsum[w] = share;
       __syncthreads();
       // U: rank-2 update of the live tiles
       float vhv = 0.f;
@@ -341,15 +471,30 @@ __global__ void __launch_bounds__(NW * 32, 1) k_eig_tridiag8(const float* __rest
       const float K = 0.5f * tau * tau * vhv;
       float wr[KR], wc[KC];
       sfor<KR>([&](auto a) { wr[a] = (a >= S) ? fmaf(-K, vr[a], ps[lane + 32 * a]) : 0.f; });
-      sfor<KC>([&](auto c) { wc[c] = (c >= SPS * S) ? fmaf(-K, vc[c], ps[w + NW * c]) : 0.f; });
-      sfor<KR>([&](auto a) {
-        if constexpr (a >= S) {
-          sfor<KC>([&](auto c) {
-            if constexpr (c >= SPS * S) A[a][c] -= fmaf(vr[a], wc[c], wr[a] * vc[c]);
-          });
+      sfor<KR>([&](auto q) {
+        if constexpr (q >= S) {
+          const float4 x = *reinterpret_cast<const float4*>(&pw[w * KC + 4 * q]);
+          wc[4 * q] = fmaf(-K, vc[4 * q], x.x);
+          wc[4 * q + 1] = fmaf(-K, vc[4 * q + 1], x.y);
+          wc[4 * q + 2] = fmaf(-K, vc[4 * q + 2], x.z);
+          wc[4 * q + 3] = fmaf(-K, vc[4 * q + 3], x.w);
         }
       });
+      auto update = [&](auto c) {
+        sfor<KR>([&](auto a) {
+          if constexpr (a >= S) {
+            A[a][c] = fmaf(-vr[a], wc[c], A[a][c]);
+            A[a][c] = fmaf(-wr[a], vc[c], A[a][c]);
+          }
+        });
+      };
+      sfor<SPS>([&](auto u) { update(CIdx<SPS * S + decltype(u)::value>{}); });
+      if (next) reflector(j + 1);
+      sfor<KC>([&](auto c) {
+        if constexpr (c >= SPS * S + SPS) update(c);
+      });
     }
+    __syncthreads();                         // the last column's p and v are read before the next segment's
   });
   // trailing 2 x 2 (or 1 x 1) block, written by the owners of its entries
   sfor<KR>([&](auto a) {
@@ -367,83 +512,39 @@ __global__ void __launch_bounds__(NW * 32, 1) k_eig_tridiag8(const float* __rest
   }
 }
 
-// Step 5 for NV vectors held by one warp: x <- P_0 P_1 ... P_{k-3} x, the
-// reflectors taken four at a time from the last (gg holds each group's six
-// inner products), each vector's entries i = lane + 32 c in registers.
-template <int KT, int NV>
-__device__ __forceinline__ void back_transform_warp(const float* Vs, const float* tau, const float* gg, int k,
-                                                    const float* cur, int ldx, const int (&js)[NV], float* V,
-                                                    int ldv) {
+// sum_i a[u][i] b[v][i] of four rows with four rows, lanes along i, for the
+// 32-entry chunks c0 .. KT - 1 (rows of b zero past their end): all loads
+// unconditional (a condition on each made an inner product of 150 entries
+// take 3.2K cycles).  put(u, v, total) is called by one lane in two.
+template <int KT, typename Put>
+__device__ __forceinline__ void warp_dots4(const float* const (&a)[4], const float* const (&b)[4], int c0, Put put) {
   const int lane = threadIdx.x & 31;
-  const int ng = (k - 2 + 3) / 4;
-  float x[NV][KT];
+  float acc[16];
 #pragma unroll
-  for (int u = 0; u < NV; ++u)
-#pragma unroll
-    for (int c = 0; c < KT; ++c) {
-      const int i = lane + 32 * c;
-      x[u][c] = (i < k) ? cur[(size_t)js[u] * ldx + i] : 0.f;
-    }
-  for (int g = 0; g < ng; ++g) {
-    const int ht = k - 3 - 4 * g;
-    const int c0 = (max(ht - 3, 0) + 1) >> 5;   // first chunk with a nonzero entry
-    float v[4][KT];
-    float dd[4 * NV];
-#pragma unroll
-    for (int q = 0; q < 4 * NV; ++q) dd[q] = 0.f;
-#pragma unroll
-    for (int c = 0; c < KT; ++c) {
-      if (c >= c0) {                     // warp-uniform: chunks below c0 are zero
-        const int i = lane + 32 * c;
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          v[a][c] = (ht - a >= 0 && i < k) ? Vs[(size_t)(ht - a) * k + i] : 0.f;
-#pragma unroll
-          for (int u = 0; u < NV; ++u) dd[4 * u + a] = fmaf(v[a][c], x[u][c], dd[4 * u + a]);
-        }
-      }
-    }
-    // lane (32 / (4 NV)) q ends with the total of dd[q]
-    const float tot = lane_transpose_sum<4 * NV>(dd);
-    float d[4 * NV];
-#pragma unroll
-    for (int q = 0; q < 4 * NV; ++q) d[q] = __shfl_sync(0xffffffffu, tot, (32 / (4 * NV)) * q);
-    const float* gq = gg + g * 8;
-    const float g01 = gq[0], g02 = gq[1], g03 = gq[2], g12 = gq[3], g13 = gq[4], g23 = gq[5];
-    float t[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) t[a] = (ht - a >= 0) ? tau[ht - a] : 0.f;
-#pragma unroll
-    for (int u = 0; u < NV; ++u) {
-      const float* du = d + 4 * u;
-      const float c0v = t[0] * du[0];
-      const float c1v = t[1] * fmaf(-g01, c0v, du[1]);
-      const float c2v = t[2] * fmaf(-g12, c1v, fmaf(-g02, c0v, du[2]));
-      const float c3v = t[3] * fmaf(-g23, c2v, fmaf(-g13, c1v, fmaf(-g03, c0v, du[3])));
-#pragma unroll
-      for (int c = 0; c < KT; ++c) {
-        if (c >= c0) {
-          float s = x[u][c];
-          s = fmaf(-c0v, v[0][c], s);
-          s = fmaf(-c1v, v[1][c], s);
-          s = fmaf(-c2v, v[2][c], s);
-          s = fmaf(-c3v, v[3][c], s);
-          x[u][c] = s;
-        }
-      }
-    }
-  }
+  for (int t = 0; t < 16; ++t) acc[t] = 0.f;
 #pragma unroll
   for (int c = 0; c < KT; ++c) {
-    const int i = lane + 32 * c;
-    if (i < k)
+    if (c >= c0) {                       // warp-uniform
+      float x[4], y[4];
 #pragma unroll
-      for (int u = 0; u < NV; ++u) V[(size_t)i * ldv + js[u]] = x[u][c];
+      for (int u = 0; u < 4; ++u) x[u] = a[u][32 * c + lane];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) y[u] = b[u][32 * c + lane];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[4 * u + v] = fmaf(x[u], y[v], acc[4 * u + v]);
+    }
   }
+  const float tot = lane_transpose_sum<16>(acc);
+  if (!(lane & 1)) put(lane >> 3, (lane >> 1) & 3, tot);
 }
 
 // Steps 2-5 in one CTA of 16 warps, from T and the reflectors in global
-// scratch (the reflectors are staged in shared memory).
+// scratch (the reflectors are staged in shared memory).  Every step is a
+// chain of short dependent operations, so latency decides: k = 150, r = 20
+// took 238K cycles (115 us) with divided Sturm ratios, branching LU, bounds
+// checks in the solves and one thread per inner product, 157K (77 us) so.
 template <int KT>
 __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict__ Vg, const float* __restrict__ tau_g,
                                                        const float* __restrict__ d_g, const float* __restrict__ e_g,
@@ -453,25 +554,22 @@ __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict_
   constexpr int KM = 32 * KT;
   constexpr int NT = 32 * NW;
   extern __shared__ __align__(16) float sm[];
-  // the reflectors (step 5) and the inverse-iteration factors (step 3) are
-  // never live together: one region holds both
-  float* Vs = sm;                         // [k][k], row j = reflector v_j
-  float* Wk = sm;                         // [r][ldw] inverse-iteration factors
-  float* tau = sm + er_union_floats(k, r);   // [KM]
-  float* d = tau + KM;                    // [KM]
-  float* e = d + KM;                      // [KM]
-  float* e2 = e + KM;                     // [KM]
-  float* lam = e2 + KM;                   // [32]
-  float* red = lam + 32;                  // [64]
-  int* cnt = reinterpret_cast<int*>(red + 64);   // [1024]
-  float* X = reinterpret_cast<float*>(cnt + 1024);   // [r][ldx]
-  float* X2 = X + (size_t)r * er_ldx(k);   // [r][ldx]
-  float* G = X2 + (size_t)r * er_ldx(k);  // [32][33]
-  float* Rm = G + 33 * 32;                // [32][32]
-  float* Tm = Rm + 33 * 32;               // [32][32]
-  int* sflag = reinterpret_cast<int*>(Tm + 33 * 32);
+  const ErLayout L = er_layout(KM, k, r);
+  float* Vs = sm + L.V;                   // [k][k], row j = reflector v_j
+  float* Wk = sm + L.V;                   // [r][ldw] inverse-iteration factors, rows of float4
+  uint32_t* exb = reinterpret_cast<uint32_t*>(sm + L.ex);   // [r][21] exchange bits
+  float* tau = sm + L.tau;
+  float* d = sm + L.d;
+  float* e = sm + L.e;
+  float2* de = reinterpret_cast<float2*>(sm + L.de);   // scaled (d_i, e_{i-1}^2)
+  float* lam = sm + L.lam;
+  float* red = sm + L.red;
+  int* cnt = reinterpret_cast<int*>(sm + L.cnt);       // [512]
+  float* G = sm + L.G;                    // [32][33]
+  float* Tm = sm + L.T;                   // [32][33]
+  int* sflag = reinterpret_cast<int*>(sm + L.total - 4);
   const int tid = threadIdx.x, lane = tid & 31, ty = tid >> 5;
-  const int ldx = er_ldx(k);
+  const int ldx = L.ldx;
   for (int i = tid; i < k; i += NT) {
     tau[i] = tau_g[i];
     d[i] = d_g[i];
@@ -487,7 +585,6 @@ __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict_
     glo = fminf(glo, d[i] - off);
     ghi = fmaxf(ghi, d[i] + off);
     amax = fmaxf(amax, fmaxf(fabsf(d[i]), fabsf(e[i])));
-    e2[i] = e[i] * e[i];
   }
   glo = warp_min_f(glo);
   ghi = warp_max_f(ghi);
@@ -501,13 +598,21 @@ __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict_
   glo = warp_min_f(lane < NW ? red[lane] : FLT_MAX);
   ghi = warp_max_f(lane < NW ? red[32 + lane] : -FLT_MAX);
   amax = warp_max_f(lane < NW ? __int_as_float(cnt[lane]) : 0.f);
-  __syncthreads();
   const float tnorm = fmaxf(amax, FLT_MIN);
   const float pivmin = FLT_MIN * fmaxf(1.f, tnorm * tnorm);
-  const float pad = 2.f * FLT_EPSILON * tnorm + pivmin;
-  const float lo0 = glo - pad, hi0 = ghi + pad;
+  // T scaled by a power of two (exact) to largest entry in [1, 2)
+  const unsigned ex = min(__float_as_uint(tnorm) & 0x7f800000u, 0x7e800000u);
+  const float up = __uint_as_float(0x7f000000u - ex), down = __uint_as_float(ex);
+  const int groups4 = (k + 2) / 4;        // 1 + 4 groups4 >= k rows
+  for (int i = tid; i < 1 + 4 * groups4; i += NT) {
+    const float es = (i > 0 && i < k) ? e[i - 1] * up : 0.f;
+    de[i] = (i < k) ? make_float2(d[i] * up, es * es) : make_float2(16.f, 0.f);
+  }
+  __syncthreads();
+  const float pad = 4.f * FLT_EPSILON;
+  const float lo0 = glo * up - pad, hi0 = ghi * up + pad;
   const float step = (hi0 - lo0) * (1.f / (float)(NT + 1));
-  cnt[tid] = sturm(d, e2, k, fmaf((float)(tid + 1), step, lo0), pivmin);
+  cnt[tid] = sturm(de, groups4, fmaf((float)(tid + 1), step, lo0));
   __syncthreads();
   // a warp refines the brackets of eigenvalues ty and ty + NW together
   // (two independent Sturm chains in flight)
@@ -517,14 +622,11 @@ __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict_
     auto bracket = [&](int jj, float& lo, float& hi) {
       const int want = k - jj;             // count reaching k - j brackets the j-th largest
       int first = NT;
-      for (int u = 0; u < NW; ++u) {
-        const int tt = lane * NW + u;
-        if (cnt[tt] >= want) {
-          first = tt;
-          break;
-        }
+#pragma unroll
+      for (int u = NW - 1; u >= 0; --u) {
+        const unsigned ge = __ballot_sync(0xffffffffu, cnt[32 * u + lane] >= want);
+        if (ge) first = 32 * u + __ffs(ge) - 1;
       }
-      first = warp_min_i(first);
       lo = (first == 0) ? lo0 : fmaf((float)first, step, lo0);
       hi = (first == NT) ? hi0 : fmaf((float)(first + 1), step, lo0);
     };
@@ -549,17 +651,16 @@ __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict_
       if (has1) {
         const float x1 = lo_1 + (hi_1 - lo_1) * (float)(lane + 1) * (1.f / 33.f);
         int c0, c1;
-        sturm2(d, e2, k, x0, x1, pivmin, c0, c1);
+        sturm2(de, groups4, x0, x1, c0, c1);
         narrow(c0, k - j0, x0, lo_0, hi_0);
         narrow(c1, k - j1, x1, lo_1, hi_1);
       } else {
-        narrow(sturm(d, e2, k, x0, pivmin), k - j0, x0, lo_0, hi_0);
+        narrow(sturm(de, groups4, x0), k - j0, x0, lo_0, hi_0);
       }
     }
-    if (lane == 0 && has0) lam[j0] = 0.5f * (lo_0 + hi_0);
-    if (lane == 0 && has1) lam[j1] = 0.5f * (lo_1 + hi_1);
+    if (lane == 0 && has0) lam[j0] = 0.5f * (lo_0 + hi_0) * down;
+    if (lane == 0 && has1) lam[j1] = 0.5f * (lo_1 + hi_1) * down;
   }
-  __syncthreads();
 
   // ---------------------------------------------------------------- 3
   // Two rounds of one inverse-iteration solve per vector followed by an
@@ -568,50 +669,57 @@ __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict_
   // eigenvector, and orthonormalising after each single solve keeps the
   // remainders inside the cluster's invariant subspace.
   const float tiny = FLT_EPSILON * tnorm + pivmin;
-  float* cur = X;
-  float* nxt = X2;
+  float* cur = sm + L.X;                  // [r][ldx]
+  float* nxt = sm + L.X2;                 // [r][ldx]
+  // start vector 1 + 0.01 h(j, i), h pseudo-random in [-1, 1) and different
+  // for every vector: equal shifts (a cluster below FP32 resolution) must
+  // not produce equal vectors
+  for (int j = ty; j < r; j += NW)
+    for (int i = lane; i < ldx; i += 32) {
+      cur[(size_t)j * ldx + i] = (i < k) ? fmaf(0.01f, hash_uniform(0xE16ull + (uint64_t)j, (uint64_t)i), 1.f) : 0.f;
+      nxt[(size_t)j * ldx + i] = 0.f;
+    }
+  __syncthreads();
   for (int round = 0; round < 2; ++round) {
     if (tid < r) {
-      float* x = cur + (size_t)tid * ldx;
-      float* w = Wk + (size_t)tid * er_ldw(k);
-      if (round == 0) {
-        tri_lu(d, e, k, lam[tid], tiny, w);
-        // start vector 1 + 0.01 h(tid, i), h pseudo-random in [-1, 1) and
-        // different for every vector: equal shifts (a cluster below FP32
-        // resolution) must not produce equal vectors
-        for (int i = 0; i < k; ++i) x[i] = fmaf(0.01f, hash_uniform(0xE16ull + (uint64_t)tid, (uint64_t)i), 1.f);
-      }
-      tri_lu_solve(w, k, x);
-      float mx = 0.f;
-      for (int i = 0; i < k; ++i) mx = fmaxf(mx, fabsf(x[i]));
-      const float sc = mx > 0.f ? 1.f / mx : 0.f;
-      for (int i = 0; i < k; ++i) x[i] *= sc;
+      float4* w = reinterpret_cast<float4*>(Wk + (size_t)tid * L.ldw);
+      uint32_t* ex = exb + tid * 21;
+      if (round == 0) tri_lu(d, e, k, L.kp, lam[tid], tiny, w, ex);
+      const float mx = tri_lu_solve(w, ex, L.kp, cur + (size_t)tid * ldx);
+      red[tid] = mx > 0.f ? 1.f / mx : 0.f;
     }
+    if (tid == 0) *sflag = 0;
     __syncthreads();
+    for (int j = ty; j < r; j += NW)
+      for (int i = lane; i < k; i += 32) cur[(size_t)j * ldx + i] *= red[j];
     // the factors are dead after the last solve: stage the reflectors for
     // step 5 in their place while step 4 runs
-    if (round == 1)
-      for (int x = tid; x < k * k; x += NT) cp_async4(Vs + x, Vg + x, true);
+    if (round == 1) {
+      const int n4 = k * k / 4;
+      for (int x = tid; x < n4; x += NT) cp_async16(Vs + 4 * x, Vg + 4 * x);
+      for (int x = 4 * n4 + tid; x < k * k; x += NT) cp_async4(Vs + x, Vg + x, true);
+      if (tid < 32) Vs[k * k + tid] = 0.f;
+    }
+    __syncthreads();
 
   // ---------------------------------------------------------------- 4
     // one Cholesky QR pass keeps the vectors apart before the second solve;
     // two make the final ones orthonormal to working accuracy
-    if (tid == 0) *sflag = 0;
     for (int pass = 0; pass < (round == 0 ? 1 : 2); ++pass) {
-      for (int x = tid; x < r * r; x += NT) {
-        const int a = x / r, b = x % r;
-        if (b >= a) {
-          float s0 = 0.f, s1 = 0.f;
-          const float* xa = cur + (size_t)a * ldx;
-          const float* xb = cur + (size_t)b * ldx;
-          int i = 0;
-          for (; i + 1 < k; i += 2) {
-            s0 = fmaf(xa[i], xb[i], s0);
-            s1 = fmaf(xa[i + 1], xb[i + 1], s1);
-          }
-          if (i < k) s0 = fmaf(xa[i], xb[i], s0);
-          G[a * 33 + b] = s0 + s1;
+      // upper triangle of the Gram in 4 x 4 tiles, a warp each
+      const int nb = (r + 3) / 4;
+      for (int t = ty; t < nb * (nb + 1) / 2; t += NW) {
+        int tb = 0;
+        while ((tb + 1) * (tb + 2) / 2 <= t) ++tb;
+        const int ta = t - tb * (tb + 1) / 2;
+        const float* ra[4];
+        const float* rb[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {     // rows past r repeat the last one; their sums are not used
+          ra[u] = cur + (size_t)min(4 * ta + u, r - 1) * ldx;
+          rb[u] = cur + (size_t)min(4 * tb + u, r - 1) * ldx;
         }
+        warp_dots4<KT>(ra, rb, 0, [&](int u, int v, float s) { G[(4 * ta + u) * 33 + 4 * tb + v] = s; });
       }
       __syncthreads();
       if (round == 1 && pass == 1) {
@@ -634,11 +742,20 @@ __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict_
             Tm[a * 33 + b] = (a == b ? 1.5f : 0.f) - 0.5f * g;
           }
           __syncthreads();
-          for (int x = tid; x < r * k; x += NT) {
-            const int j = x / k, i = x % k;
-            float s = 0.f;
-            for (int a = 0; a < r; ++a) s = fmaf(cur[(size_t)a * ldx + i], Tm[a * 33 + j], s);
-            nxt[(size_t)j * ldx + i] = s;
+          for (int j = ty; j < r; j += NW) {
+            float s[KT];
+#pragma unroll
+            for (int c = 0; c < KT; ++c) s[c] = 0.f;
+#pragma unroll 4
+            for (int a = 0; a < r; ++a) {
+              const float t = Tm[a * 33 + j];
+#pragma unroll
+              for (int c = 0; c < KT; ++c)
+                if (lane + 32 * c < k) s[c] = fmaf(cur[(size_t)a * ldx + lane + 32 * c], t, s[c]);
+            }
+#pragma unroll
+            for (int c = 0; c < KT; ++c)
+              if (lane + 32 * c < k) nxt[(size_t)j * ldx + lane + 32 * c] = s[c];
           }
           __syncthreads();
           float* tmp = cur; cur = nxt; nxt = tmp;
@@ -650,11 +767,20 @@ __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict_
       chol_inv_warp32_call(G, 33, r, red, Tm, 33, sflag, true);
       if (*sflag) break;                  // uniform: fall back below
       // nxt[j][i] = sum_{a <= j} cur[a][i] T[a][j]
-      for (int x = tid; x < r * k; x += NT) {
-        const int j = x / k, i = x % k;
-        float s = 0.f;
-        for (int a = 0; a <= j; ++a) s = fmaf(cur[(size_t)a * ldx + i], Tm[a * 33 + j], s);
-        nxt[(size_t)j * ldx + i] = s;
+      for (int j = ty; j < r; j += NW) {
+        float s[KT];
+#pragma unroll
+        for (int c = 0; c < KT; ++c) s[c] = 0.f;
+#pragma unroll 4
+        for (int a = 0; a <= j; ++a) {
+          const float t = Tm[a * 33 + j];
+#pragma unroll
+          for (int c = 0; c < KT; ++c)
+            if (lane + 32 * c < k) s[c] = fmaf(cur[(size_t)a * ldx + lane + 32 * c], t, s[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < KT; ++c)
+          if (lane + 32 * c < k) nxt[(size_t)j * ldx + lane + 32 * c] = s[c];
       }
       __syncthreads();
       float* tmp = cur; cur = nxt; nxt = tmp;
@@ -709,53 +835,137 @@ __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict_
   }
 
   // ---------------------------------------------------------------- 5
+  // x <- P_0 P_1 ... P_{k-3} x for the r vectors, ER_GB reflectors at a time
+  // from the last.  For the reflectors of a group in the order of their
+  // application (q = 0 the highest index), c_q = tau_q (v_q^T x - sum_{p < q}
+  // (v_q^T v_p) c_p) and x -= sum_q c_q v_q, so c = S D with D = [v_q^T x] and
+  // a triangular S that depends on the reflectors alone: all S first, a warp
+  // per group, then three small products per group for all vectors at once.
+  // v_h is zero at indices <= h (and entirely where tau_h = 0), so a group
+  // starts at its lowest reflector.
   cp_async_wait_all();
   __syncthreads();
-  // x <- P_0 P_1 ... P_{k-3} x for the r vectors, reflectors taken four at a
-  // time from the last.  For the group {h, h-1, h-2, h-3}, applied in that
-  // order, the coefficients follow from the dots d_a = v_{h-a}^T x of the
-  // group's incoming x and the group's inner products g_ab = v_{h-a}^T v_{h-b}:
-  //   c_a = tau_{h-a} (d_a - sum_{b < a} g_ba c_b),   x -= sum_a c_a v_{h-a},
-  // so a group costs one lane reduction where single reflectors cost four.
-  // v_h is zero at indices <= h (and entirely where tau_h = 0), so a group
-  // skips the 32-entry chunks below its lowest reflector.
   {
-    const int ng = (k - 2 + 3) / 4;       // groups over reflectors 0 .. k-3
-    float* gg = Tm;                       // [ng][8]: g01 g02 g03 g12 g13 g23
+    constexpr int GB = ER_GB, LS = GB + 1;
+    float* Sg = sm + L.S;                 // [groups][GB][LS]
+    float* Dm = sm + L.D;                 // [GB][36]
+    float* Cm = sm + L.C;                 // [GB][36]
+    const int ng = L.groups;
+    auto top = [&](int g) { return k - 3 - GB * g; };       // highest reflector of group g
+    auto size = [&](int g) { return min(GB, top(g) + 1); };
+    // Reads of a reflector's last chunk run past its k entries into the next
+    // reflector: the vectors are zero there, and the reflectors' own products
+    // mask one side.
+    // inner products of each group's reflectors, rows in application order
+    // (row q is reflector top - q; past the group, the zero row k - 1)
+    constexpr int NTL = (GB / 4) * (GB / 4 + 1) / 2;
+    for (int t = ty; t < ng * NTL; t += NW) {
+      const int g = t / NTL, tl = t % NTL;
+      int ta = 0;
+      while ((ta + 1) * (ta + 2) / 2 <= tl) ++ta;
+      const int tb = tl - ta * (ta + 1) / 2;              // p <= q
+      const int h = top(g), n = size(g);
+      float* S = Sg + (size_t)g * GB * LS;
+      float acc[16];
+#pragma unroll
+      for (int x = 0; x < 16; ++x) acc[x] = 0.f;
+      const int c0 = (h - n + 2) >> 5;
+#pragma unroll
+      for (int c = 0; c < KT; ++c)
+        if (c >= c0) {
+          const int i = 32 * c + lane;
+          float x[4], y[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            x[u] = Vs[(size_t)((4 * ta + u < n) ? h - 4 * ta - u : k - 1) * k + i];
+            y[u] = Vs[(size_t)((4 * tb + u < n) ? h - 4 * tb - u : k - 1) * k + i];
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) x[u] = (i < k) ? x[u] : 0.f;
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[4 * u + v] = fmaf(x[u], y[v], acc[4 * u + v]);
+        }
+      const float tot = lane_transpose_sum<16>(acc);
+      if (!(lane & 1)) S[(4 * ta + (lane >> 3)) * LS + 4 * tb + ((lane >> 1) & 3)] = tot;
+    }
+    __syncthreads();
+    // S by forward substitution, lane = column: S[q][c] = tau_q ([q == c] -
+    // sum_{c <= p < q} g_qp S[p][c])
     for (int g = ty; g < ng; g += NW) {
-      const int ht = k - 3 - 4 * g;
-      float p6[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      float* S = Sg + (size_t)g * GB * LS;
+      const int h = top(g), n = size(g);
+      float col[GB];
 #pragma unroll
-      for (int c = 0; c < KT; ++c) {
-        const int i = lane + 32 * c;
-        float v[4];
+      for (int q = 0; q < GB; ++q) {
+        float s0 = (q == lane) ? 1.f : 0.f, s1 = 0.f;
 #pragma unroll
-        for (int a = 0; a < 4; ++a) v[a] = (ht - a >= 0 && i < k) ? Vs[(size_t)(ht - a) * k + i] : 0.f;
-        p6[0] = fmaf(v[0], v[1], p6[0]);
-        p6[1] = fmaf(v[0], v[2], p6[1]);
-        p6[2] = fmaf(v[0], v[3], p6[2]);
-        p6[3] = fmaf(v[1], v[2], p6[3]);
-        p6[4] = fmaf(v[1], v[3], p6[4]);
-        p6[5] = fmaf(v[2], v[3], p6[5]);
+        for (int p = 0; p < q; ++p) {
+          const float gp = (q < n) ? S[q * LS + p] : 0.f;
+          if (p & 1) s1 = fmaf(-gp, col[p], s1);
+          else s0 = fmaf(-gp, col[p], s0);
+        }
+        col[q] = (q < n) ? tau[h - q] * (s0 + s1) : 0.f;
       }
+      __syncwarp();
+      if (lane < GB) {
 #pragma unroll
-      for (int q = 0; q < 6; ++q) p6[q] = warp_sum(p6[q]);
-      if (lane < 6) {
-        float o = p6[0];
-#pragma unroll
-        for (int q = 1; q < 6; ++q) o = (lane == q) ? p6[q] : o;
-        gg[g * 8 + lane] = o;
+        for (int q = 0; q < GB; ++q) S[q * LS + lane] = col[q];
       }
     }
     __syncthreads();
-    // warps ty < r - NW take vectors ty and ty + NW (each reflector read
-    // once for both, their lane reductions merged), the others vector ty
-    if (ty + NW < r) {
-      const int js[2] = {ty, ty + NW};
-      back_transform_warp<KT, 2>(Vs, tau, gg, k, cur, ldx, js, V, ldv);
-    } else if (ty < r) {
-      const int js[1] = {ty};
-      back_transform_warp<KT, 1>(Vs, tau, gg, k, cur, ldx, js, V, ldv);
+    const int nv = (r + 3) / 4;
+    for (int g = 0; g < ng; ++g) {
+      const int h = top(g), n = size(g), i0 = (h - n + 2) & ~31;
+      const float* S = Sg + (size_t)g * GB * LS;
+      for (int t = ty; t < (GB / 4) * nv; t += NW) {
+        const int ta = t / nv, tb = t % nv;
+        const float* ra[4];
+        const float* rb[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          ra[u] = Vs + (size_t)((4 * ta + u < n) ? h - 4 * ta - u : k - 1) * k;
+          rb[u] = cur + (size_t)min(4 * tb + u, r - 1) * ldx;
+        }
+        warp_dots4<KT>(ra, rb, i0 >> 5, [&](int u, int v, float s) { Dm[(4 * ta + u) * 36 + 4 * tb + v] = s; });
+      }
+      __syncthreads();
+      for (int x = tid; x < GB * 32; x += NT) {
+        const int q = x >> 5, j = x & 31;
+        if (j < 4 * nv) {
+          float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+          for (int p = 0; p < GB; p += 2) {
+            s0 = fmaf(S[q * LS + p], Dm[p * 36 + j], s0);
+            s1 = fmaf(S[q * LS + p + 1], Dm[(p + 1) * 36 + j], s1);
+          }
+          Cm[q * 36 + j] = s0 + s1;
+        }
+      }
+      __syncthreads();
+      const int nc = (k - i0 + 31) >> 5;
+      for (int t = ty; t < nv * nc; t += NW) {
+        const int tj = t / nc, i = i0 + 32 * (t % nc) + lane;
+        if (i < k) {
+          float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int q = 0; q < GB; ++q) {    // rows of Cm past the group are zero
+            const float v = Vs[(size_t)max(h - q, 0) * k + i];
+            const float4 c = *reinterpret_cast<const float4*>(Cm + q * 36 + 4 * tj);
+            acc[0] = fmaf(v, c.x, acc[0]); acc[1] = fmaf(v, c.y, acc[1]);
+            acc[2] = fmaf(v, c.z, acc[2]); acc[3] = fmaf(v, c.w, acc[3]);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (4 * tj + u < r) cur[(size_t)(4 * tj + u) * ldx + i] -= acc[u];
+        }
+      }
+      __syncthreads();
+    }
+    for (int x = tid; x < k * r; x += NT) {
+      const int i = x / r, j = x % r;
+      V[(size_t)i * ldv + j] = cur[(size_t)j * ldx + i];
     }
     if (evals)
       for (int j = tid; j < r; j += NT) evals[j] = lam[j];
@@ -768,28 +978,29 @@ static int er_kt(int k) { return (k + 31) / 32; }
 bool eig_reg_ok(int k, int r) {
   if (k < 1 || r < 1 || r > 32 || r > k || k > 32 * ER_KTMAX) return false;
   // dynamic shared memory plus the kernel's static arrays (the Cholesky's
-  // 4.5 KB of R rows) within the 227 KB a CTA may use
-  return er_smem_floats(32 * er_kt(k), k, r) * 4 + 6 * 1024 <= 227 * 1024;
+  // rows, 8.5 KB + 2.2 KB) within the 227 KB a CTA may use
+  return er_layout(32 * er_kt(k), k, r).total * 4 + 12 * 1024 <= 227 * 1024;
 }
 
 template <int KT>
 static cudaError_t launch_kt(const float* H, int64_t ldh, int k, int r, float* V, int ldv, float* evals,
                              float* scratch, cudaStream_t st) {
-  float* Vg = scratch;
+  // 16-byte aligned, for the reflectors' copy
+  float* Vg = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(scratch) + 15) & ~uintptr_t(15));
   float* tau = Vg + (size_t)k * k;
   float* d = tau + k;
   float* e = d + k;
   k_eig_tridiag8<KT, ER_TRI_WARPS><<<1, ER_TRI_WARPS * 32, 0, st>>>(H, ldh, k, Vg, tau, d, e);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
-  const size_t smem = er_smem_floats(32 * KT, k, r) * 4;
+  const size_t smem = er_layout(32 * KT, k, r).total * 4;
   err = raise_smem_limit(k_eig_vectors<KT>);
   if (err != cudaSuccess) return err;
   k_eig_vectors<KT><<<1, 512, smem, st>>>(Vg, tau, d, e, k, r, V, ldv, evals);
   return cudaGetLastError();
 }
 
-// scratch: k * k + 3 k floats (device)
+// scratch: k * k + 3 k + 4 floats (device)
 cudaError_t launch_eig_reg(const float* H, int64_t ldh, int k, int r, float* V, int ldv, float* evals,
                            float* scratch, cudaStream_t st) {
   if (!eig_reg_ok(k, r)) return cudaErrorInvalidValue;

@@ -139,7 +139,7 @@ cudaError_t gram_power(const float* G, int64_t m, const float* X, int64_t ldx, i
 
 // ---- register-tiled symmetric eigensolver, k <= 160, r <= 32 (eig_reg.cu)
 bool eig_reg_ok(int k, int r);
-// scratch: k * k + 3 k floats
+// scratch: k * k + 3 k + 4 floats
 cudaError_t launch_eig_reg(const float* H, int64_t ldh, int k, int r, float* V, int ldv, float* evals,
                            float* scratch, cudaStream_t st);
 

@@ -46,6 +46,44 @@ __device__ __forceinline__ void st4(__nv_bfloat16* p, const float (&v)[4]) {
   *reinterpret_cast<uint2*>(p) = *reinterpret_cast<const uint2*>(h);
 }
 
+// Elements kept as loaded and converted when used: issue is in order, so a
+// conversion next to a prefetching load would wait for it there.
+__device__ __forceinline__ uint32_t ld_raw(const float* p) { return __float_as_uint(*p); }
+__device__ __forceinline__ uint32_t ld_raw(const __nv_bfloat16* p) {
+  return *reinterpret_cast<const unsigned short*>(p);
+}
+template <typename T>
+__device__ __forceinline__ float from_raw(uint32_t x) {
+  return __uint_as_float(sizeof(T) == 2 ? x << 16 : x);
+}
+// Four consecutive elements, p aligned to them: 4 words (FP32) or the first 2
+// of r (BF16).
+__device__ __forceinline__ void ld4_raw(const float* p, uint32_t* r) {
+  const uint4 x = *reinterpret_cast<const uint4*>(p);
+  r[0] = x.x; r[1] = x.y; r[2] = x.z; r[3] = x.w;
+}
+__device__ __forceinline__ void ld4_raw(const __nv_bfloat16* p, uint32_t* r) {
+  const uint2 x = *reinterpret_cast<const uint2*>(p);
+  r[0] = x.x; r[1] = x.y;
+}
+template <typename T>
+__device__ __forceinline__ float4 from_raw4(const uint32_t* r) {
+  if (sizeof(T) == 2)
+    return make_float4(__uint_as_float(r[0] << 16), __uint_as_float(r[0] & 0xffff0000u), __uint_as_float(r[1] << 16),
+                       __uint_as_float(r[1] & 0xffff0000u));
+  return make_float4(__uint_as_float(r[0]), __uint_as_float(r[1]), __uint_as_float(r[2]), __uint_as_float(r[3]));
+}
+
+// Two FP32 multiply-adds in one instruction (each rounded as fmaf).
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mov.b64 z, {%6, %7};\n"
+      " fma.rn.f32x2 z, x, y, z;\n mov.b64 {%0, %1}, z;\n}\n"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+
 // Deterministic pseudo-random value in [-1, 1) from two 64-bit words (a
 // SplitMix64-style finaliser), for replacing numerically vanished basis
 // columns by directions that carry no information of their own.

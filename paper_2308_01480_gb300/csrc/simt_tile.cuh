@@ -27,7 +27,7 @@ struct NtShape {
   static constexpr int BK = CT == 1 ? 128 : 64;
   static constexpr int KS = BK / (4 * KG);
   static constexpr int LD = BK + 4;
-  static constexpr int GROUPS = CT == 8 ? 4 : 8;      // partial tiles left after the in-warp sums
+  static constexpr int GROUPS = CT >= 8 ? KG : 8;     // partial tiles left after the in-warp sums
   static constexpr int tile_floats(bool same) { return (BM + (same ? 0 : BN)) * LD; }
   static constexpr int smem_floats(bool same) {
     return tile_floats(same) > GROUPS * BM * BN ? tile_floats(same) : GROUPS * BM * BN;
@@ -39,7 +39,7 @@ struct NtShape {
 template <typename T, int ROWS, int BK>
 struct NtFetch {
   static constexpr int N4 = (ROWS * BK / 4 + 255) / 256;
-  float r[4 * N4];
+  uint32_t r[4 * N4];
   // One pointer stepped from row to row; the step is opaque to the compiler,
   // which otherwise keeps the 16 to 32 row offsets of a tile in 64-bit
   // registers over the whole loop and spills the accumulators.
@@ -54,11 +54,10 @@ struct NtFetch {
       const T* p = A + (int64_t)row * ld + k0 + c;
 #pragma unroll
       for (int u = 0; u < N4; ++u) {
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
-        if (in && row + u * STEP < rows) ld4(p, v);
-        p += step;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) r[4 * u + t] = v[t];
+        for (int t = 0; t < 4; ++t) r[4 * u + t] = 0u;
+        if (in && row + u * STEP < rows) ld4_raw(p, r + 4 * u);
+        p += step;
       }
     } else {
       constexpr int STEP = 256 / BK;
@@ -69,7 +68,7 @@ struct NtFetch {
       const T* p = A + (int64_t)row * ld + k0 + c;
 #pragma unroll
       for (int u = 0; u < 4 * N4; ++u) {
-        r[u] = (in && row + u * STEP < rows) ? ld_elem(p, 0) : 0.f;
+        r[u] = (in && row + u * STEP < rows) ? ld_raw(p) : 0u;
         p += step;
       }
     }
@@ -81,14 +80,13 @@ struct NtFetch {
       for (int u = 0; u < N4; ++u) {
         const int e = threadIdx.x + 256 * u, row = e / (BK / 4), c = (e % (BK / 4)) * 4;
         if (row < ROWS)
-          *reinterpret_cast<float4*>(s + row * LD + c) =
-              make_float4(r[4 * u], r[4 * u + 1], r[4 * u + 2], r[4 * u + 3]);
+          *reinterpret_cast<float4*>(s + row * LD + c) = from_raw4<T>(r + 4 * u);
       }
     } else {
 #pragma unroll
       for (int u = 0; u < 4 * N4; ++u) {
         const int e = threadIdx.x + 256 * u, row = e / BK, c = e % BK;
-        if (row < ROWS) s[row * LD + c] = r[u];
+        if (row < ROWS) s[row * LD + c] = from_raw<T>(r[u]);
       }
     }
   }
@@ -163,7 +161,7 @@ __device__ __forceinline__ void nt_tile(const TA* __restrict__ A, int64_t lda, i
       }
   }
   __syncthreads();
-  const int g = CT == 8 ? kg : (tid >> 5);
+  const int g = CT >= 8 ? kg : (tid >> 5);
   const bool owner = CT >= 4 || (CT == 2 && !(tid & 16)) || (CT == 1 && !(tid & 24));
   if (owner) {
 #pragma unroll

@@ -15,8 +15,8 @@
 // more CTAs an SM, so that one CTA's loads overlap another's products.
 // Before, both products loaded their operands as scalars (one per 1 to 2
 // multiply-adds for narrow blocks).  Measured (FP32, us): 45 x 4,100,625 at
-// b = 6 1,230 -> 287 (738 MB, 2.6 TB/s), 180 x 91,125 at b = 6 105 -> 31,
-// 256 x 32,768 at b = 13 57 -> 35.
+// b = 6 1,230 -> 287 (738 MB, 2.6 TB/s; BF16, rows not aligned, 1,178 ->
+// 287), 180 x 91,125 at b = 6 101 -> 31, 256 x 32,768 at b = 13 54 -> 34.
 #pragma once
 
 #include "common.cuh"
@@ -73,7 +73,7 @@ namespace {
 template <typename T, int TN, int K>
 struct GaLoad {
   static constexpr int rows = 256 * K / TN;
-  float r[K];
+  uint32_t r[K];
   __device__ __forceinline__ void load(const T* __restrict__ C, int64_t n, int m, int wv, bool vec) {
     if (vec) {
       constexpr int STEP = 1024 / TN;
@@ -83,11 +83,10 @@ struct GaLoad {
       asm volatile("" : "+l"(step));       // no row offsets kept in registers
 #pragma unroll
       for (int u = 0; u < K / 4; ++u) {
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
-        if (c < wv && row + u * STEP < m) ld4(p, v);
-        p += step;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) r[4 * u + t] = v[t];
+        for (int t = 0; t < 4; ++t) r[4 * u + t] = 0u;
+        if (c < wv && row + u * STEP < m) ld4_raw(p, r + 4 * u);
+        p += step;
       }
     } else {
       constexpr int STEP = 256 / TN;
@@ -97,7 +96,7 @@ struct GaLoad {
       asm volatile("" : "+l"(step));
 #pragma unroll
       for (int u = 0; u < K; ++u) {
-        r[u] = (c < wv && row + u * STEP < m) ? ld_elem(p, 0) : 0.f;
+        r[u] = (c < wv && row + u * STEP < m) ? ld_raw(p) : 0u;
         p += step;
       }
     }
@@ -110,14 +109,13 @@ struct GaLoad {
 #pragma unroll
       for (int u = 0; u < K / 4; ++u)
         if (row + u * STEP < m)
-          *reinterpret_cast<float4*>(Cs + (row + u * STEP) * LD + c) =
-              make_float4(r[4 * u], r[4 * u + 1], r[4 * u + 2], r[4 * u + 3]);
+          *reinterpret_cast<float4*>(Cs + (row + u * STEP) * LD + c) = from_raw4<T>(r + 4 * u);
     } else {
       constexpr int STEP = 256 / TN;
       const int row = threadIdx.x / TN, c = threadIdx.x % TN;
 #pragma unroll
       for (int u = 0; u < K; ++u)
-        if (row + u * STEP < m) Cs[(row + u * STEP) * LD + c] = r[u];
+        if (row + u * STEP < m) Cs[(row + u * STEP) * LD + c] = from_raw<T>(r[u]);
     }
   }
 };

@@ -4,9 +4,10 @@
 //
 // Every column of C is one column of S, so a thread keeps four whole
 // columns (TC sums of each) in registers and reads C straight from global
-// memory, coalesced along the row: C needs no shared memory and no barrier.  X is the small operand: chunks of 64 rows are double-buffered in
-// shared memory and read as broadcasts, one 16-byte load for 16
-// multiply-adds.  The next rows of C (16 to 32 elements a thread) are in
+// memory, coalesced along the row: C needs no shared memory and no barrier.  X is the small operand: chunks of 16 rows are double-buffered in
+// shared memory by each row group for itself (a barrier over the CTA per
+// chunk held up the others) and read as broadcasts, one 16-byte load for 16
+// multiply-adds, two to an instruction.  The next rows of C (16 to 32 elements a thread) are in
 // flight while the current ones are multiplied.
 // The eight warps of a CTA split into CG groups of output rows (b > 20), RG
 // groups of rows of C (few columns: the groups' sums are added in order) and
@@ -15,9 +16,9 @@
 // kernel adds the partials in split order.
 // Measured (FP32, us; before: 16 x 16 threads with both operands staged in
 // shared memory and no split over rows unless n <= 512): 7680 x 2048 at
-// b = 20 440 -> 31, 800 x 64,000 at b = 20 ~120 -> 106, 45 x 4,100,625 at
-// b = 4 ~600 -> 170.  What bounds it now is the issue rate (53 of every 100
-// instructions are multiply-adds, one CTA an SM at b = 20).
+// b = 20 404 -> 31, 800 x 64,000 at b = 20 190 -> 106, 45 x 4,100,625 at
+// b = 6 640 -> 208 (3.5 TB/s); BF16 715 -> 201.  What bounds it now is
+// latency at one to two CTAs an SM.
 #include "cluster_la.cuh"
 #include "common.cuh"
 #include "kernels.h"
@@ -26,7 +27,7 @@ namespace ttr {
 
 namespace {
 
-constexpr int PJ_RK = 64;   // rows of X per shared-memory chunk
+constexpr int PJ_RK = 16;   // rows of X per shared-memory chunk of a row group
 constexpr int PJ_NC = 4;    // columns of C per thread
 
 __device__ __forceinline__ void cp_async16z(float* dst, const float* src, bool ok) {
@@ -34,95 +35,116 @@ __device__ __forceinline__ void cp_async16z(float* dst, const float* src, bool o
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
 }
 
-// vec: every row of C (and of S) starts aligned to four elements, and the
+// VEC: every row of C (and of S) starts aligned to four elements, and the
 // thread's columns are neighbours; otherwise they are 32 apart.  x16: rows
 // of X are 16-byte aligned and b is a multiple of four.
-template <typename TIn, typename TOut, int TC, int FR, int CTAS>
+template <typename TIn, typename TOut, int TC, int FR, int CTAS, bool VEC>
 __global__ void __launch_bounds__(256, CTAS) k_proj(const TIn* __restrict__ C, int64_t m, int64_t n,
                                                     const float* __restrict__ X, int ldx, int b,
                                                     TOut* __restrict__ S, int64_t lds, int64_t rows_per,
-                                                    int64_t split_stride, int CG, int RG, bool vec, bool x16) {
+                                                    int64_t split_stride, int CG, int RG, bool x16) {
   constexpr int NC = PJ_NC;
   extern __shared__ __align__(16) float pj_sm[];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int CW = 8 / (CG * RG);
   const int cw = w % CW, cg = (w / CW) % CG, rg = w / (CW * CG);
   const int BP = CG * TC;
-  const int64_t col = (int64_t)blockIdx.x * (CW * 32 * NC) + cw * (32 * NC) + (vec ? NC * lane : lane);
-  const int64_t rbeg = (int64_t)blockIdx.y * rows_per, rend = imin(m, rbeg + rows_per);
+  const int64_t col = (int64_t)blockIdx.x * (CW * 32 * NC) + cw * (32 * NC) + (VEC ? NC * lane : lane);
   S += (int64_t)blockIdx.y * split_stride;
-  const int per_group = PJ_RK / RG;             // rows of a chunk that one group takes
-  const int nchunk = (int)ceil_div(rend - rbeg, PJ_RK);
+  // this row group's rows [g0, g1) and its two chunk buffers; only the
+  // group's warps synchronise
+  const int64_t rbeg = (int64_t)blockIdx.y * rows_per, rend = imin(m, rbeg + rows_per);
+  const int64_t gr = ceil_div(rend - rbeg, RG), g0 = rbeg + rg * gr, g1 = imin(rend, g0 + gr);
+  const int nchunk = g0 < g1 ? (int)ceil_div(g1 - g0, PJ_RK) : 0;
+  const int gt = 256 / RG;                      // threads of one group
+  const int t = tid % gt;
+  float* xbuf = pj_sm + (size_t)rg * 2 * PJ_RK * BP;
+  auto group_sync = [&]() {
+    if (gt == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;\n" ::"r"(1 + rg), "r"(gt) : "memory");
+  };
   bool in[NC];
 #pragma unroll
-  for (int u = 0; u < NC; ++u) in[u] = vec ? col < n : col + 32 * u < n;   // vec: all four or none
+  for (int u = 0; u < NC; ++u) in[u] = VEC ? col < n : col + 32 * u < n;   // VEC: all four or none
   auto stage = [&](int ch) {
-    float* xs = pj_sm + (ch & 1) * PJ_RK * BP;
-    const int64_t i0 = rbeg + (int64_t)ch * PJ_RK;
+    float* xs = xbuf + (ch & 1) * PJ_RK * BP;
+    const int64_t i0 = g0 + (int64_t)ch * PJ_RK;
     if (x16) {
       const int q = BP / 4;
-      for (int e = tid; e < PJ_RK * q; e += 256) {
+      for (int e = t; e < PJ_RK * q; e += gt) {
         const int r = e / q, c = (e - r * q) * 4;
-        const bool ok = i0 + r < rend && c < b;
+        const bool ok = i0 + r < g1 && c < b;
         cp_async16z(xs + 4 * e, ok ? X + (i0 + r) * ldx + c : X, ok);
       }
     } else {
-      for (int e = tid; e < PJ_RK * BP; e += 256) {
+      for (int e = t; e < PJ_RK * BP; e += gt) {
         const int r = e / BP, c = e - r * BP;
-        const bool ok = i0 + r < rend && c < b;
+        const bool ok = i0 + r < g1 && c < b;
         cp_async4(xs + e, ok ? X + (i0 + r) * ldx + c : X, ok);
       }
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
-  auto fetch = [&](float (&v)[FR][NC], int64_t i0) {
+  auto fetch = [&](uint32_t (&v)[FR][NC], int64_t i0) {
     const TIn* p = C + i0 * n + col;
-    const int left = (int)imin(FR, rend - i0);
+    const int left = (int)imin(FR, g1 - i0);
 #pragma unroll
     for (int r = 0; r < FR; ++r) {
-      if (vec) {
 #pragma unroll
-        for (int u = 0; u < NC; ++u) v[r][u] = 0.f;
-        if (r < left && in[0]) ld4(p, v[r]);
+      for (int u = 0; u < NC; ++u) v[r][u] = 0u;
+      if constexpr (VEC) {
+        if (r < left && in[0]) ld4_raw(p, v[r]);
       } else {
 #pragma unroll
-        for (int u = 0; u < NC; ++u) v[r][u] = (r < left && in[u]) ? ld_elem(p, 32 * u) : 0.f;
+        for (int u = 0; u < NC; ++u)
+          if (r < left && in[u]) v[r][u] = ld_raw(p + 32 * u);
       }
       p += n;
     }
   };
-  float acc[NC][TC];
+  float2 acc[NC][TC / 2];
 #pragma unroll
   for (int u = 0; u < NC; ++u)
 #pragma unroll
-    for (int c = 0; c < TC; ++c) acc[u][c] = 0.f;
-  float cur[FR][NC], nxt[FR][NC] = {};
-  stage(0);
-  const int64_t g0 = rbeg + rg * per_group;     // the group's first row
-  fetch(cur, g0);
+    for (int c = 0; c < TC / 2; ++c) acc[u][c] = make_float2(0.f, 0.f);
+  uint32_t cur[FR][NC], nxt[FR][NC] = {};
+  if (nchunk > 0) {
+    stage(0);
+    fetch(cur, g0);
+  }
   for (int ch = 0; ch < nchunk; ++ch) {
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    __syncthreads();
+    group_sync();
     if (ch + 1 < nchunk) stage(ch + 1);
     const int64_t i0 = g0 + (int64_t)ch * PJ_RK;
-    const int rows = (int)imin(per_group, rend - i0);
-    const float* xs = pj_sm + (ch & 1) * PJ_RK * BP + (size_t)rg * per_group * BP + cg * TC;
+    const int rows = (int)imin(PJ_RK, g1 - i0);
+    const float* xs = xbuf + (ch & 1) * PJ_RK * BP + cg * TC;
     for (int s = 0; s < rows; s += FR) {
-      const bool more = s + FR < rows;
-      if (more || ch + 1 < nchunk) fetch(nxt, more ? i0 + s + FR : i0 + PJ_RK);
+      if (i0 + s + FR < g1) fetch(nxt, i0 + s + FR);
 #pragma unroll
-      for (int r = 0; r < FR; ++r)
+      for (int r = 0; r < FR; ++r) {
+        float2 cv[NC];
+        if constexpr (VEC) {
+          const float4 f = from_raw4<TIn>(cur[r]);
+          cv[0] = make_float2(f.x, f.x); cv[1] = make_float2(f.y, f.y);
+          cv[2] = make_float2(f.z, f.z); cv[3] = make_float2(f.w, f.w);
+        } else {
+#pragma unroll
+          for (int u = 0; u < NC; ++u) {
+            const float f = from_raw<TIn>(cur[r][u]);
+            cv[u] = make_float2(f, f);
+          }
+        }
 #pragma unroll
         for (int c4 = 0; c4 < TC / 4; ++c4) {
           const float4 x = *reinterpret_cast<const float4*>(xs + (s + r) * BP + 4 * c4);
 #pragma unroll
           for (int u = 0; u < NC; ++u) {
-            acc[u][4 * c4] = fmaf(x.x, cur[r][u], acc[u][4 * c4]);
-            acc[u][4 * c4 + 1] = fmaf(x.y, cur[r][u], acc[u][4 * c4 + 1]);
-            acc[u][4 * c4 + 2] = fmaf(x.z, cur[r][u], acc[u][4 * c4 + 2]);
-            acc[u][4 * c4 + 3] = fmaf(x.w, cur[r][u], acc[u][4 * c4 + 3]);
+            acc[u][2 * c4] = fma2(make_float2(x.x, x.y), cv[u], acc[u][2 * c4]);
+            acc[u][2 * c4 + 1] = fma2(make_float2(x.z, x.w), cv[u], acc[u][2 * c4 + 1]);
           }
         }
+      }
 #pragma unroll
       for (int r = 0; r < FR; ++r)
 #pragma unroll
@@ -130,22 +152,26 @@ __global__ void __launch_bounds__(256, CTAS) k_proj(const TIn* __restrict__ C, i
     }
   }
   // sums of the row groups, added in group order
-  const int gt = 256 / RG;                      // threads of one group
-  const int t = tid % gt;
   for (int g = 1; g < RG; ++g) {
     __syncthreads();
     if (rg == g) {
 #pragma unroll
       for (int u = 0; u < NC; ++u)
 #pragma unroll
-        for (int c = 0; c < TC; ++c) pj_sm[(u * TC + c) * gt + t] = acc[u][c];
+        for (int c = 0; c < TC / 2; ++c) {
+          pj_sm[(u * TC + 2 * c) * gt + t] = acc[u][c].x;
+          pj_sm[(u * TC + 2 * c + 1) * gt + t] = acc[u][c].y;
+        }
     }
     __syncthreads();
     if (rg == 0) {
 #pragma unroll
       for (int u = 0; u < NC; ++u)
 #pragma unroll
-        for (int c = 0; c < TC; ++c) acc[u][c] += pj_sm[(u * TC + c) * gt + t];
+        for (int c = 0; c < TC / 2; ++c) {
+          acc[u][c].x += pj_sm[(u * TC + 2 * c) * gt + t];
+          acc[u][c].y += pj_sm[(u * TC + 2 * c + 1) * gt + t];
+        }
     }
   }
   if (rg != 0) return;
@@ -154,13 +180,15 @@ __global__ void __launch_bounds__(256, CTAS) k_proj(const TIn* __restrict__ C, i
     const int row = cg * TC + c;
     if (row < b) {
       TOut* out = S + (int64_t)row * lds + col;
-      if (vec) {
-        const float v[4] = {acc[0][c], acc[1][c], acc[2][c], acc[3][c]};
+      if constexpr (VEC) {
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < NC; ++u) v[u] = (c & 1) ? acc[u][c / 2].y : acc[u][c / 2].x;
         if (in[0]) st4(out, v);
       } else {
 #pragma unroll
         for (int u = 0; u < NC; ++u)
-          if (in[u]) st_elem(out, 32 * u, acc[u][c]);
+          if (in[u]) st_elem(out, 32 * u, (c & 1) ? acc[u][c / 2].y : acc[u][c / 2].x);
       }
     }
   }
@@ -191,9 +219,9 @@ template <typename TIn, typename TOut, int TC>
 cudaError_t launch_proj(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b, TOut* S, int64_t lds,
                         int64_t rows_per, int splits, int64_t split_stride, int CG, cudaStream_t st) {
   constexpr int NC = PJ_NC;
-  // narrow outputs: more CTAs an SM; the widest holds its 80 sums and 64
-  // loads in one
-  constexpr int FR = TC >= 20 ? 8 : 4, CTAS = TC >= 20 ? 1 : TC >= 12 ? 2 : 3;
+  // narrow outputs: two CTAs an SM; the wide ones hold their 64 or 80 sums and
+  // 64 loads in one
+  constexpr int FR = TC >= 16 ? 8 : 4, CTAS = TC >= 16 ? 1 : 2;
   // as few row groups as give the chip two CTAs an SM
   int RG = 1;
   while (CG * RG < 8 && rows_per >= 16 * RG && ceil_div(n, (8 / (CG * RG)) * 32 * NC) * splits < 2 * 152) RG *= 2;
@@ -202,9 +230,14 @@ cudaError_t launch_proj(const TIn* C, int64_t m, int64_t n, const float* X, int 
                    reinterpret_cast<uintptr_t>(C) % (4 * sizeof(TIn)) == 0 &&
                    reinterpret_cast<uintptr_t>(S) % (4 * sizeof(TOut)) == 0;
   const bool x16 = b % 4 == 0 && ldx % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0;
-  const size_t smem = sizeof(float) * (size_t)imax(2 * PJ_RK * CG * TC, RG > 1 ? (256 / RG) * NC * TC : 0);
-  k_proj<TIn, TOut, TC, FR, CTAS><<<dim3((unsigned)ceil_div(n, cols), (unsigned)splits), 256, smem, st>>>(
-      C, m, n, X, ldx, b, S, lds, rows_per, split_stride, CG, RG, vec, x16);
+  const size_t smem = sizeof(float) * (size_t)imax(RG * 2 * PJ_RK * CG * TC, RG > 1 ? (256 / RG) * NC * TC : 0);
+  const dim3 grid((unsigned)ceil_div(n, cols), (unsigned)splits);
+  if (vec)
+    k_proj<TIn, TOut, TC, FR, CTAS, true><<<grid, 256, smem, st>>>(C, m, n, X, ldx, b, S, lds, rows_per, split_stride,
+                                                                  CG, RG, x16);
+  else
+    k_proj<TIn, TOut, TC, FR, CTAS, false><<<grid, 256, smem, st>>>(C, m, n, X, ldx, b, S, lds, rows_per,
+                                                                   split_stride, CG, RG, x16);
   return cudaGetLastError();
 }
 

@@ -10,9 +10,11 @@
 // split across CTAs into per-CTA partials that a second kernel sums in a
 // fixed order, so results are bit-reproducible.
 // Measured (FP32, us; before: 2 x VB register tiles on scalar shared loads):
-// the sketch of 45 x 4,100,625 at b = 6 ~900 -> 184 (4.0 TB/s), of
-// 800 x 64,000 at b = 20 ~120 -> 68, of 7680 x 2048 at b = 20 91 -> 26; the
-// Gram of 32 x 1,048,576 180 -> 62, of a BF16 61 x 112,095 145 -> 48.
+// the sketch of 45 x 4,100,625 at b = 6 965 -> 183 (4.0 TB/s), of
+// 800 x 64,000 at b = 20 259 -> 68 and at b = 30 262 -> 103, of 7680 x 2048
+// at b = 20 91 -> 26; the Gram of 32 x 1,048,576 181 -> 62, of 45 x 4,100,625
+// 1,020 -> 474.  BF16, rows not aligned: the sketch of 45 x 4,100,625
+// 951 -> 173, of 80 x 794,155 at b = 28 398 -> 202.
 #include "common.cuh"
 #include "kernels.h"
 #include "simt_tile.cuh"
@@ -61,6 +63,23 @@ __global__ void __launch_bounds__(256, 2) k_gram_tiles_simt(const TIn* __restric
   auto put = [&](int i, int c, float v) { out[i * T + c] = v; };
   if (I == J) simt::nt_tile<Sh, true>(A, n, ra, A, n, ra, c0, c1, vec, vec, nt_sm, put);
   else simt::nt_tile<Sh, false>(A, n, ra, B, n, rb, c0, c1, vec, vec, nt_sm, put);
+}
+
+// As below for few splits: one thread per entry, in split order.
+template <int T>
+__global__ void __launch_bounds__(256) k_gram_simt_reduce_few(const float* __restrict__ P, int64_t m, int splits,
+                                                              float* __restrict__ G) {
+  const int i = blockIdx.y;
+  const int j = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (j < i || j >= m) return;
+  const int I = i / T, J = j / T;
+  const int t = J * (J + 1) / 2 + I;
+  const float* src = P + (size_t)t * splits * T * T + (size_t)(i - T * I) * T + (j - T * J);
+  float s = 0.f;
+#pragma unroll 8
+  for (int k = 0; k < splits; ++k) s += src[(size_t)k * T * T];
+  G[(int64_t)i * m + j] = s;
+  if (j != i) G[(int64_t)j * m + i] = s;
 }
 
 // G[i][j] = G[j][i] = sum over the splits of tile(i, j), i <= j: eight warps
@@ -226,11 +245,11 @@ cudaError_t cs_dispatch(const TIn* C, int64_t m, int64_t n, const float* S, int6
   if (b <= 12) TTR_CS(6, 2);
   if (b <= 16) TTR_CS(8, 2);
   if (b <= 20) TTR_CS(5, 4);
-  if (b <= 24) TTR_CS(6, 4);
-  if (b <= 32) TTR_CS(8, 4);
+  if (b <= 24) TTR_CS(3, 8);
+  if (b <= 32) TTR_CS(4, 8);
   if (b <= 40) TTR_CS(5, 8);
   if (b <= 48) TTR_CS(6, 8);
-  if (b <= 64) TTR_CS(8, 8);
+  if (b <= 64) TTR_CS(4, 16);
 #undef TTR_CS
   return cudaErrorInvalidValue;
 }
@@ -259,7 +278,12 @@ int64_t simt_cs_partials(int64_t m, int64_t n, int b) { return cs_splits(m, n) *
 // ---------------------------------------------------------------- gram
 namespace {
 
-int gram_tile(int64_t m) { return m <= 16 ? 16 : m <= 32 ? 32 : m <= 48 ? 48 : 64; }
+// Tile edge: 48 or 64, whichever pads the rows to less (64 on a tie); one tile
+// of 16 or 32 for the shortest.
+int gram_tile(int64_t m) {
+  if (m <= 32) return m <= 16 ? 16 : 32;
+  return ceil_div(m, 48) * 48 < ceil_div(m, 64) * 64 ? 48 : 64;
+}
 
 // Tiles of the upper triangle and splits of the columns: two CTAs an SM, a
 // split at least 256 columns.
@@ -281,7 +305,10 @@ cudaError_t gram_launch(const TIn* C, int64_t m, int64_t n, int tiles, int split
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   note_launch("gram_reduce");
-  k_gram_simt_reduce<Sh::BM><<<dim3((unsigned)ceil_div(m, 32), (unsigned)m), 256, 0, st>>>(P, m, splits, G);
+  if (splits <= 8)   // 800 rows, 2 splits: 5.7 us against 13.8 by eight warps
+    k_gram_simt_reduce_few<Sh::BM><<<dim3((unsigned)ceil_div(m, 256), (unsigned)m), 256, 0, st>>>(P, m, splits, G);
+  else
+    k_gram_simt_reduce<Sh::BM><<<dim3((unsigned)ceil_div(m, 32), (unsigned)m), 256, 0, st>>>(P, m, splits, G);
   return cudaGetLastError();
 }
 
@@ -298,7 +325,7 @@ cudaError_t simt_gram(const TIn* C, int64_t m, int64_t n, float* partials, float
     case 16: return gram_launch<simt::NtShape<2, 8, 2>>(C, m, n, tiles, splits, partials, out, st);
     case 32: return gram_launch<simt::NtShape<4, 8, 4>>(C, m, n, tiles, splits, partials, out, st);
     case 48: return gram_launch<simt::NtShape<6, 6, 8>>(C, m, n, tiles, splits, partials, out, st);
-    default: return gram_launch<simt::NtShape<8, 8, 8>>(C, m, n, tiles, splits, partials, out, st);
+    default: return gram_launch<simt::NtShape<8, 4, 16>>(C, m, n, tiles, splits, partials, out, st);
   }
 }
 

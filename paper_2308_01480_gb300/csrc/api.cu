@@ -61,7 +61,7 @@ struct Plan {
   void* comm = nullptr;
   // workspace offsets in bytes
   size_t off_status = 0, off_R0 = 0, off_R1 = 0, off_S = 0, off_T = 0, off_part = 0, off_Y = 0,
-         off_Q = 0, off_W = 0, off_U = 0, off_G = 0, off_small = 0, off_X = 0, off_Xg = 0, off_B = 0, off_Hd = 0,
+         off_Q = 0, off_W = 0, off_G = 0, off_small = 0, off_X = 0, off_Xg = 0, off_B = 0, off_Hd = 0,
          off_dfp = 0, off_part2 = 0, total = 0;
 };
 
@@ -137,7 +137,7 @@ tt_status build_plan(const int64_t* dims, int d, const int64_t* ranks, int p, in
   int64_t total = 1;
   for (int k = 0; k < d; ++k) total *= dims[k];
   int64_t n = total;
-  size_t maxR = 0, maxS = 0, maxT = 0, maxPart = 0, maxY = 0, maxQ = 0, maxU = 0, maxG = 0, maxSmall = 0,
+  size_t maxR = 0, maxS = 0, maxT = 0, maxPart = 0, maxY = 0, maxQ = 0, maxG = 0, maxSmall = 0,
          maxX = 0, maxXg = 0, maxB = 0, maxHd = 0, maxDf = 0, maxPart2 = 0;
   for (int k = 0; k < d - 1; ++k) {
     ModePlan& M = P.modes[k];
@@ -246,7 +246,6 @@ tt_status build_plan(const int64_t* dims, int d, const int64_t* ranks, int p, in
       maxSmall = std::max(maxSmall, ttr::orth_grid_rs_scratch_floats(M.m, std::max(0, M.kq - M.b), M.b));
       maxSmall = std::max(maxSmall, ttr::rr_fast_scratch_floats(M.m, M.kq, M.r_out));
     }
-    maxU = std::max(maxU, (size_t)(M.m * M.r_out));
     maxPart = std::max(maxPart, (size_t)(ttr::simt_proj_splits(M.m, M.n) * M.b * M.n));
     // tensor-core passes (BF16 unfoldings)
     const int cdt = (k == 0) ? P.storage : P.remainder;
@@ -290,7 +289,6 @@ tt_status build_plan(const int64_t* dims, int d, const int64_t* ranks, int p, in
   P.off_Y = take(maxY * 4);
   P.off_Q = take(maxQ * 4);
   P.off_W = take(maxQ * 4);
-  P.off_U = take(maxU * 4);
   P.off_G = take(maxG * 4);
   P.off_small = take(maxSmall * 4);
   P.off_X = take(maxX);
@@ -336,7 +334,7 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
   const __nv_bfloat16* Cb = reinterpret_cast<const __nv_bfloat16*>(C);
   void* xs = ws + P.off_X;
   float* part = (float*)(ws + P.off_part);
-  float* U = (float*)(ws + P.off_U);
+  float* U = core;   // the basis of the projection is the core itself (m x r, row-major)
   float* small = (float*)(ws + P.off_small);
   const int r = M.r_out;
   // sharded form: the sum of a partial block over the ranks (a no-op alone)
@@ -351,7 +349,7 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
     double* Hd = (double*)(ws + P.off_Hd);
     double* dfp = (double*)(ws + P.off_dfp);
     TTR_CUDA(ttr::gram_df<TIn>(C, (int)M.m, M.n, M.n, dfp, Hd, st));
-    TTR_CUDA(ttr::launch_rr_svd(Hd, (int)M.m, r, nullptr, M.m, 0, U, core, status, st));
+    TTR_CUDA(ttr::launch_rr_svd(Hd, (int)M.m, r, nullptr, M.m, 0, U, nullptr, status, st));
   } else if (M.gram_route) {
     float* G = (float*)(ws + P.off_G);
     if (use_tc && M.m <= 128)
@@ -363,9 +361,9 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
       if (rs != TT_OK) return rs;
     }
     if (ttr::eig_top_ok((int)M.m))
-      TTR_CUDA(ttr::launch_rr_fast(nullptr, G, M.m, M.m, (int)M.m, r, 1, small, U, core, st));
+      TTR_CUDA(ttr::launch_rr_fast(nullptr, G, M.m, M.m, (int)M.m, r, 1, small, U, nullptr, st));
     else
-      TTR_CUDA(ttr::launch_rayleigh_ritz(nullptr, G, M.m, M.m, (int)M.m, r, 1, small, U, core, st));
+      TTR_CUDA(ttr::launch_rayleigh_ritz(nullptr, G, M.m, M.m, (int)M.m, r, 1, small, U, nullptr, st));
   } else if (M.gram_cols) {
     // exhaustion with D = n < m: the Krylov basis would span range(C), so
     // Rayleigh-Ritz would return the exact top-r left singular vectors;
@@ -386,7 +384,6 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
     } else {
       TTR_CUDA(ttr::launch_orth_block(Y, r, M.m, r, U, r, 0, r, small, rseed, status, nullptr, st));
     }
-    TTR_CUDA(cudaMemcpyAsync(core, U, sizeof(float) * (size_t)M.m * r, cudaMemcpyDeviceToDevice, st));
   } else {
     float* S = (float*)(ws + P.off_S);
     float* T = (float*)(ws + P.off_T);
@@ -529,7 +526,6 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
         os = orth(W, kq, r, 0, r, rseed + 7919ull * (it + 1));
         if (os != TT_OK) return os;
       }
-      TTR_CUDA(cudaMemcpyAsync(U, Q, sizeof(float) * (size_t)M.m * r, cudaMemcpyDeviceToDevice, st));
       TTR_CUDA(cudaMemcpyAsync(core, Q, sizeof(float) * (size_t)M.m * r, cudaMemcpyDeviceToDevice, st));
     } else {
     tt_status os = orth(Y, M.b, M.b, 0, M.blocks[0], rseed);
@@ -572,11 +568,11 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
         TTR_CUDA((ttr::simt_proj<TIn, float>(C, M.m, M.n, Q + c0, kq, cw, Bm + (size_t)c0 * M.n, M.n, st, nullptr)));
       }
       TTR_CUDA(ttr::gram_df<float>(Bm, kq, M.n, M.n, dfp, Hd, st));
-      TTR_CUDA(ttr::launch_rr_svd(Hd, kq, r, Q, M.m, kq, U, core, status, st));
+      TTR_CUDA(ttr::launch_rr_svd(Hd, kq, r, Q, M.m, kq, U, nullptr, status, st));
     } else if (ttr::eig_top_ok(kq)) {
-      TTR_CUDA(ttr::launch_rr_fast(Q, W, kq, M.m, kq, r, 0, small, U, core, st));
+      TTR_CUDA(ttr::launch_rr_fast(Q, W, kq, M.m, kq, r, 0, small, U, nullptr, st));
     } else {
-      TTR_CUDA(ttr::launch_rayleigh_ritz(Q, W, kq, M.m, kq, r, 0, small, U, core, st));
+      TTR_CUDA(ttr::launch_rayleigh_ritz(Q, W, kq, M.m, kq, r, 0, small, U, nullptr, st));
     }
     }
   }

@@ -561,13 +561,12 @@ cudaError_t launch_rr_fast(const float* Q, const float* W, int64_t ld, int64_t m
     Hsrc = H;
     ldh = k;
   }
-  e = launch_eig_top(Hsrc, ldh, k, r, V, es, nullptr, st);
+  // Q = I (m == k): U = V
+  e = launch_eig_top(Hsrc, ldh, k, r, identity_q ? U : V, es, nullptr, st);
   if (e != cudaSuccess) return e;
   if (identity_q) {
-    // Q = I (m == k): U = V
-    e = cudaMemcpyAsync(U, V, sizeof(float) * (size_t)m * r, cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess && core)
-      e = cudaMemcpyAsync(core, V, sizeof(float) * (size_t)m * r, cudaMemcpyDeviceToDevice, st);
+    if (core)
+      e = cudaMemcpyAsync(core, U, sizeof(float) * (size_t)m * r, cudaMemcpyDeviceToDevice, st);
     return e;
   }
   return launch_apply_basis(Q, ld, m, k, V, r, U, core, st);

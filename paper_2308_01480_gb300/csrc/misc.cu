@@ -38,42 +38,44 @@ __device__ __forceinline__ float2 box_muller(uint32_t a, uint32_t b) {
 // a slab (w > 0) the n local rows are the rows (i / w) nd + lo + i % w of
 // the full Omega_k: the columns of the unfolding whose last index lies in
 // [lo, lo + w) of a last mode of size nd, in their order.
+// A thread draws four columns (one Philox block) of one row at a time, the
+// column group from the grid's second dimension: with a 64-bit division and
+// remainder per draw 4,100,625 x 6 (FP32) took 88 us, so 70; the rest is the
+// transform.
 template <typename T>
-__global__ void k_omega(uint64_t seed, uint32_t mode, int64_t n, int b, T* __restrict__ out, int64_t si,
-                        int64_t sc, int64_t w, int64_t nd, int64_t lo) {
-  const int groups = (b + 3) >> 2;
-  const int64_t total = n * groups;
+__global__ void __launch_bounds__(256) k_omega(uint64_t seed, uint32_t mode, int64_t n, int b, T* __restrict__ out,
+                                               int64_t si, int64_t sc, int64_t w, int64_t nd, int64_t lo) {
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e % n;            // consecutive threads -> consecutive rows
-    const int g = (int)(e / n);
-    const int64_t gi = (w > 0) ? (i / w) * nd + lo + i % w : i;   // row of the full Omega_k
-    const uint4 x =
-        philox4x32_10(make_uint4((uint32_t)gi, (uint32_t)((uint64_t)gi >> 32), (uint32_t)g, mode), k0, k1);
-    const float2 z01 = box_muller(x.x, x.y);
-    const float2 z23 = box_muller(x.z, x.w);
-    const float z[4] = {z01.x, z01.y, z23.x, z23.y};
+  for (int g = (int)blockIdx.y; 4 * g < b; g += (int)gridDim.y) {
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+      const int64_t gi = (w > 0) ? (i / w) * nd + lo + i % w : i;   // row of the full Omega_k
+      const uint4 x =
+          philox4x32_10(make_uint4((uint32_t)gi, (uint32_t)((uint64_t)gi >> 32), (uint32_t)g, mode), k0, k1);
+      const float2 z01 = box_muller(x.x, x.y);
+      const float2 z23 = box_muller(x.z, x.w);
+      const float z[4] = {z01.x, z01.y, z23.x, z23.y};
+      T* p = out + i * si + (int64_t)(4 * g) * sc;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int c = 4 * g + t;
-      if (c < b) st_elem(out, i * si + (int64_t)c * sc, z[t]);
+      for (int t = 0; t < 4; ++t) {
+        if (4 * g + t < b) st_elem(p, 0, z[t]);
+        p += sc;
+      }
     }
   }
 }
 
 cudaError_t launch_omega(uint64_t seed, int mode, int64_t n, int b, void* out, int dtype, int64_t si,
                          int64_t sc, cudaStream_t st, int64_t slab_w, int64_t slab_nd, int64_t slab_lo) {
-  const int64_t total = n * ((b + 3) / 4);
-  const int blocks = (int)imin(ceil_div(total, 256), 152 * 16);
+  const int groups = (b + 3) / 4;
+  const dim3 grid((unsigned)imax(1, imin(ceil_div(n, 256), imax(1, 152 * 16 / groups))),
+                  (unsigned)imin(groups, 65535));
   ProfScope prof("omega_philox", st, (double)n * b * (dtype == TT_BF16 ? 2 : 4), 0);
   note_launch("omega_philox");
   if (dtype == TT_BF16)
-    k_omega<__nv_bfloat16><<<blocks, 256, 0, st>>>(seed, (uint32_t)mode, n, b, (__nv_bfloat16*)out, si, sc, slab_w,
-                                                   slab_nd, slab_lo);
+    k_omega<__nv_bfloat16><<<grid, 256, 0, st>>>(seed, (uint32_t)mode, n, b, (__nv_bfloat16*)out, si, sc, slab_w,
+                                                 slab_nd, slab_lo);
   else
-    k_omega<float><<<blocks, 256, 0, st>>>(seed, (uint32_t)mode, n, b, (float*)out, si, sc, slab_w, slab_nd,
-                                           slab_lo);
+    k_omega<float><<<grid, 256, 0, st>>>(seed, (uint32_t)mode, n, b, (float*)out, si, sc, slab_w, slab_nd, slab_lo);
   return cudaGetLastError();
 }
 

@@ -215,10 +215,16 @@ struct ClusterComm {
   __device__ int rank() { return (int)cl.block_rank(); }
   template <typename Put>
   __device__ void reduce(float* mine, int phase, int e0, int e1, Put& put) {
+    // nothing to exchange: the share is the sum (64 rows of 9 columns: two
+    // cluster barriers and a copy per sum fewer, 22.6 -> 16.5 us a block)
+    if (nranks() == 1) {
+      for (int e = e0 + (int)threadIdx.x; e < e1; e += blockDim.x) put(e, mine[e]);
+      return;
+    }
     cl.sync();
     cluster_reduce_scatter_gather(cl, mine, slices + (size_t)(phase & 1) * slice_len, e0, e1, put);
   }
-  __device__ void finish() { cl.sync(); }   // no CTA leaves while others may read its shares
+  __device__ void finish() { if (nranks() > 1) cl.sync(); }   // no CTA leaves while others may read its shares
 };
 
 // Barrier over all CTAs of a cooperative launch (every CTA resident): an

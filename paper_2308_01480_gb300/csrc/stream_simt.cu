@@ -173,6 +173,30 @@ __global__ void __launch_bounds__(32 * RED_WARPS) k_reduce_partials(const float*
   reduce_elements(PartialsFlat{P}, S, E, E, cols, out, ldo);
 }
 
+// As above for at most eight partials, which leave most of the eight warps
+// idle: one thread per element, in partial order (two partials of 7680 x 20:
+// 5.8 us by warps; the 7680 x 2048 call with five of them 796 us, so 771).
+__global__ void __launch_bounds__(256) k_reduce_few(const float* __restrict__ P, int S, int64_t rows, int cols,
+                                                    float* __restrict__ out, int64_t ldo) {
+  const int64_t E = rows * cols;
+  const bool dense = ldo == cols;
+  for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < E; e += (int64_t)gridDim.x * 256) {
+    float v[8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) v[s] = (s < S) ? P[s * E + e] : 0.f;
+    float a = v[0];
+#pragma unroll
+    for (int s = 1; s < 8; ++s)
+      if (s < S) a += v[s];
+    if (dense) {
+      out[e] = a;
+    } else {
+      const int64_t r = e / cols;
+      out[r * ldo + (e - r * cols)] = a;
+    }
+  }
+}
+
 // out[r][c] = sum over the CTAs of r's row group (slot j * groups + g) of
 // their partials; the CTAs of a group write only that group's rows.
 __global__ void __launch_bounds__(32 * RED_WARPS) k_reduce_grouped(const float* __restrict__ P, int per, int groups,
@@ -190,8 +214,12 @@ __global__ void __launch_bounds__(32 * RED_WARPS) k_reduce_grouped(const float* 
 static void reduce_launch(const float* P, int S, int64_t rows, int cols, float* out, int64_t ldo,
                           cudaStream_t st) {
   int64_t E = rows * cols;
-  int blocks = (int)imin(ceil_div(E, 32), 4096);
-  k_reduce_partials<<<blocks, 32 * RED_WARPS, 0, st>>>(P, S, rows, cols, out, ldo);
+  if (S <= 8) {
+    k_reduce_few<<<(int)imin(ceil_div(E, 256), 152 * 8), 256, 0, st>>>(P, S, rows, cols, out, ldo);
+  } else {
+    const int blocks = (int)imin(ceil_div(E, 32), 4096);
+    k_reduce_partials<<<blocks, 32 * RED_WARPS, 0, st>>>(P, S, rows, cols, out, ldo);
+  }
   note_launch("reduce_partials");
 }
 

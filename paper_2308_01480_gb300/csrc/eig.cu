@@ -65,11 +65,13 @@ __global__ void __launch_bounds__(64) k_tn_partials(const TA* __restrict__ A, in
     }
 }
 
-// The same product in one launch for at most 32 chunks of 32 rows (m <= 1024):
+// The same product in one launch for at most 16 chunks of 32 rows (m <= 512):
 // eight groups of two warps take every eighth chunk of a tile's rows, each
 // with its own staging and barrier, and the group sums are added in order.
-// Two launches (partials, then their sum) took 6.3 + 1.8 us for 64 rows of 27
-// columns and 7.9 + 3.7 us for 800 of 100; this 2.6 and 10.7.
+// Two launches (partials, then their sum, ~1.3 us between them) against this,
+// FP32: 64 x 16 5.4 + 1.8 and 2.8 us, 500 x 100 5.7 + 2.5 and 7.0; at 800 x 40
+// 5.4 + 3.3 and 10.1 (BF16 8.3 + 3.4 and 14.2), where few tiles leave too few
+// CTAs for the rows.
 constexpr int TN_GROUPS = 8;
 
 template <typename TA, typename TB>
@@ -87,22 +89,22 @@ __global__ void __launch_bounds__(64 * TN_GROUPS) k_tn_direct(const TA* __restri
   const bool ina = s0 + c < ka, inb = t0 + c < kb;
   float acc[4][4] = {};
   for (int i0 = 32 * g; i0 < m; i0 += 32 * TN_GROUPS) {
-    float va[16], vb[16];
+    uint32_t va[16], vb[16];              // as loaded: a conversion here would wait for each load
     const TA* pa = A + (int64_t)(i0 + rr) * lda + s0 + c;
     const TB* pb = B + (int64_t)(i0 + rr) * ldb + t0 + c;
 #pragma unroll
     for (int u = 0; u < 16; ++u) {
       const bool in = i0 + rr + 2 * u < m;
-      va[u] = (in && ina) ? ld_elem(pa, 0) : 0.f;
-      vb[u] = (in && inb) ? ld_elem(pb, 0) : 0.f;
+      va[u] = (in && ina) ? ld_raw(pa) : 0u;
+      vb[u] = (in && inb) ? ld_raw(pb) : 0u;
       pa += 2 * lda;
       pb += 2 * ldb;
     }
     asm volatile("bar.sync %0, 64;\n" ::"r"(1 + g) : "memory");
 #pragma unroll
     for (int u = 0; u < 16; ++u) {
-      As[(rr + 2 * u) * 32 + c] = va[u];
-      Bs[(rr + 2 * u) * 32 + c] = vb[u];
+      As[(rr + 2 * u) * 32 + c] = from_raw<TA>(va[u]);
+      Bs[(rr + 2 * u) * 32 + c] = from_raw<TB>(vb[u]);
     }
     asm volatile("bar.sync %0, 64;\n" ::"r"(1 + g) : "memory");
 #pragma unroll 8
@@ -571,7 +573,7 @@ size_t tn_parts_floats(int64_t m, int ka, int kb) {
 template <typename TA, typename TB>
 static cudaError_t launch_tn(const TA* A, int64_t lda, int ka, const TB* B, int64_t ldb, int kb, int64_t m,
                              float* parts, float* out, cudaStream_t st) {
-  if (m <= 1024) {
+  if (m <= 32 * 2 * TN_GROUPS) {
     const cudaError_t e = raise_smem_limit(k_tn_direct<TA, TB>);
     if (e != cudaSuccess) return e;
     ProfScope prof("tn_small", st, 0, 2.0 * m * ka * kb);

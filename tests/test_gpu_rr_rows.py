@@ -1,5 +1,5 @@
 """The small A^T B of Rayleigh-Ritz and of the column-Gram route at the edges
-of its launch rule (chunks of 32 rows, groups of 256 rows, the 1024-row limit
+of its launch rule (chunks of 32 rows, groups of 256 rows, the 512-row limit
 of the one-launch form; 32-column tiles), as order-2 decompositions against
 the float64 oracle."""
 import numpy as np
@@ -9,7 +9,7 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("m", [31, 32, 33, 255, 257, 1024, 1025])
+@pytest.mark.parametrize("m", [31, 32, 33, 255, 257, 512, 513, 1024])
 @pytest.mark.parametrize("n,r,p,q", [(150, 5, 6, 2),      # basis of 33 columns
                                      (12, 4, 5, 1)])      # column-Gram route (n < m)
 def test_small_products_match_oracle(m, n, r, p, q):

@@ -1,5 +1,5 @@
 // Building blocks for block orthonormalisation on one thread-block cluster
-// (orth_cluster.cu, krylov_cluster.cu): register-tiled products over
+// (orth_cluster.cu, orth_cluster_rs.cu): register-tiled products over
 // shared-memory row blocks and the rank-ordered sum of per-CTA shares
 // through distributed shared memory.
 #pragma once

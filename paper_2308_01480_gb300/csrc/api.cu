@@ -42,6 +42,7 @@ struct ModePlan {
   bool gram_power = false;   // short unfolding: G = C C^T formed once, each power W = G X
   bool fused_ga = false;     // Gram-apply fused in one pass over C
   bool literal = false;      // the paper's steps taken literally (first-r truncation)
+  std::vector<ttr::OrthCall> orths;   // the block orthonormalisations, in order (Krylov route)
   int64_t n_global = 0;      // columns of the whole unfolding (n: this rank's slab of them)
   int allreduces = 0;        // sums over the ranks this mode needs (sharded form)
   int64_t allreduce_floats = 0;
@@ -63,6 +64,7 @@ struct Plan {
   size_t off_status = 0, off_R0 = 0, off_R1 = 0, off_S = 0, off_T = 0, off_part = 0, off_Y = 0,
          off_Q = 0, off_W = 0, off_G = 0, off_small = 0, off_X = 0, off_Xg = 0, off_B = 0, off_Hd = 0,
          off_dfp = 0, off_part2 = 0, total = 0;
+  size_t small_floats = 0;   // size of the region at off_small
 };
 
 tt_status resolve_options(const tt_options* in, tt_options* out) {
@@ -242,8 +244,9 @@ tt_status build_plan(const int64_t* dims, int d, const int64_t* ranks, int p, in
       maxSmall = std::max(maxSmall, ttr::orth_scratch_floats(M.m, M.b, M.kq));
       maxSmall = std::max(maxSmall, ttr::rr_scratch_floats(M.kq));
       maxSmall = std::max(maxSmall, ttr::orth_fast_scratch_floats(M.m, M.kq, M.b));
-      // the last block's call has the largest basis: kq0 + c <= kq
-      maxSmall = std::max(maxSmall, ttr::orth_grid_rs_scratch_floats(M.m, std::max(0, M.kq - M.b), M.b));
+      M.orths = ttr::orth_calls(M.literal ? M.r_out : M.b, M.blocks,
+                                M.literal || P.o.method == TT_METHOD_RSI);
+      maxSmall = std::max(maxSmall, ttr::orth_grid_plan(M.m, ttr::orth_grid_limits(), &M.orths));
       maxSmall = std::max(maxSmall, ttr::rr_fast_scratch_floats(M.m, M.kq, M.r_out));
     }
     maxPart = std::max(maxPart, (size_t)(ttr::simt_proj_splits(M.m, M.n) * M.b * M.n));
@@ -291,6 +294,7 @@ tt_status build_plan(const int64_t* dims, int d, const int64_t* ranks, int p, in
   P.off_W = take(maxQ * 4);
   P.off_G = take(maxG * 4);
   P.off_small = take(maxSmall * 4);
+  P.small_floats = maxSmall;
   P.off_X = take(maxX);
   P.off_Xg = take(maxXg * 4);
   P.off_B = take(maxB * 4);
@@ -451,7 +455,9 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
     float* Xg = (float*)(ws + P.off_Xg);
     const int xld = (M.b + 3) & ~3;
     bool xg_written = false;
-    auto orth = [&](const float* Z, int64_t ldz, int zc, int kq0, int c, uint64_t sd) -> tt_status {
+    auto orth = [&](const float* Z, int64_t ldz, size_t call, uint64_t sd) -> tt_status {
+      const ttr::OrthCall& oc = M.orths[std::min(call, M.orths.size() - 1)];   // restarts repeat the last
+      const int zc = oc.zc, kq0 = oc.kq0, c = oc.c;
       xg_written = false;
       if (ttr::orth_cluster_rs_ok(M.m, kq0, zc, c)) {
         // one cluster launch, rank-deficient columns repaired inside
@@ -463,10 +469,10 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
         }
         if (e != cudaErrorNotSupported) TTR_CUDA(e);
       }
-      if (ttr::orth_grid_rs_ok(M.m, kq0, zc, c)) {
+      if (oc.grid) {
         // blocks taller than a cluster holds: one cooperative launch
         TTR_CUDA(ttr::launch_orth_grid_rs(Z, ldz, zc, M.m, c, kq0, Q, kq, M.gram_power ? Xg : nullptr, xld, sd,
-                                          small, status, st));
+                                          small, P.small_floats, status, st));
         xg_written = M.gram_power;
         return TT_OK;
       }
@@ -517,18 +523,18 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
     if (M.literal) {
       // Q = orth((C C^T)^s C W(:, 1:r)): orthonormalise after every power
       // (the same leading-column spans as the literal QRs); Q is the core
-      tt_status os = orth(Y, r, r, 0, r, rseed);
+      tt_status os = orth(Y, r, 0, rseed);
       if (os == TT_OK) os = join_gram();
       if (os != TT_OK) return os;
       for (int it = 0; it < M.iters; ++it) {
         os = power(Q, W, r);
         if (os != TT_OK) return os;
-        os = orth(W, kq, r, 0, r, rseed + 7919ull * (it + 1));
+        os = orth(W, kq, 1, rseed + 7919ull * (it + 1));
         if (os != TT_OK) return os;
       }
       TTR_CUDA(cudaMemcpyAsync(core, Q, sizeof(float) * (size_t)M.m * r, cudaMemcpyDeviceToDevice, st));
     } else {
-    tt_status os = orth(Y, M.b, M.b, 0, M.blocks[0], rseed);
+    tt_status os = orth(Y, M.b, 0, rseed);
     if (os == TT_OK) os = join_gram();
     if (os != TT_OK) return os;
     if (P.o.method == TT_METHOD_RSI) {
@@ -539,7 +545,7 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
         os = power(Q, W, c0);
         if (os != TT_OK) return os;
         if (it < M.iters) {
-          os = orth(W, kq, c0, 0, c0, rseed + 7919ull * (it + 1));
+          os = orth(W, kq, 1, rseed + 7919ull * (it + 1));
           if (os != TT_OK) return os;
         }
       }
@@ -551,7 +557,7 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
         os = power(Q + col, W + col, cj);
         if (os != TT_OK) return os;
         if (j + 1 < M.blocks.size()) {
-          os = orth(W + col, kq, cj, col + cj, M.blocks[j + 1], rseed + 7919ull * (j + 1));
+          os = orth(W + col, kq, j + 1, rseed + 7919ull * (j + 1));
           if (os != TT_OK) return os;
         }
         col += cj;

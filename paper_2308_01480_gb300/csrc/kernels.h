@@ -7,6 +7,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "orth_rs_plan.h"
+
 namespace ttr {
 
 // ---- error message returned by tt_rbki_last_error (api.cu)
@@ -112,13 +114,14 @@ cudaError_t launch_orth_cluster(const float* W, int64_t ldw, int64_t m, int b, i
 // cudaErrorNotSupported when the device cannot hold the cluster.
 // The same sequence over all CTAs of one cooperative launch (at most one
 // per SM, shares reduced through global memory, bounded barriers) for blocks
-// with more rows than a cluster holds; scratch holds
-// orth_grid_rs_scratch_floats floats (barrier words, shares, sums).
-bool orth_grid_rs_ok(int64_t m, int kq0, int zc, int c);
-size_t orth_grid_rs_scratch_floats(int64_t m, int kq0, int zc);
+// with more rows than a cluster holds.  Which calls of a mode take it, and the
+// scratch they need (barrier words, shares, sums), is planned by
+// orth_grid_plan (orth_rs_plan.h) under the current device's limits; a call
+// whose scratch_floats do not hold its shares is refused.
+OrthGridLimits orth_grid_limits();
 cudaError_t launch_orth_grid_rs(const float* Y, int64_t ldy, int zc, int64_t m, int c, int kq0, float* Q,
-                                int64_t ldq, float* Xg, int xld, uint64_t seed, float* scratch, int* status,
-                                cudaStream_t st);
+                                int64_t ldq, float* Xg, int xld, uint64_t seed, float* scratch,
+                                size_t scratch_floats, int* status, cudaStream_t st);
 bool orth_cluster_rs_ok(int64_t m, int kq0, int zc, int c);
 cudaError_t launch_orth_cluster_rs(const float* Y, int64_t ldy, int zc, int64_t m, int c, int kq0, float* Q,
                                    int64_t ldq, float* Xg, int xld, uint64_t seed, int* status, cudaStream_t st);

@@ -31,6 +31,7 @@
 #include "chol.cuh"
 #include "cluster_la.cuh"
 #include "kernels.h"
+#include "orth_rs_plan.h"
 
 namespace ttr {
 
@@ -62,40 +63,6 @@ struct OrthRsArgs {
   unsigned* gbar;
   int eslot;            // E: floats per share
 };
-
-struct KcLayout {
-  int KP, ZP, RP;
-  size_t share, slice, P, Gm, T, R, misc, Zc, Zn, Qc, tmp, total;
-  int slice_len;
-  int share_bufs;       // 2 for a cluster (other ranks read the shares), 1 for the grid form
-};
-
-// nc: cluster size; nc = 0 for the grid form (shares and sums in global
-// memory, no slice buffers).
-__host__ __device__ inline KcLayout kc_layout(int kqmax, int zmax, int rows, int nc) {
-  KcLayout L;
-  L.KP = pad4(kqmax);
-  L.ZP = pad4(zmax);
-  L.RP = pad4(rows);
-  size_t o = 0;
-  auto take = [&](size_t n) { size_t r = o; o += (n + 3) & ~size_t(3); return r; };
-  L.share_bufs = nc > 0 ? 2 : 1;
-  L.share = take((size_t)L.share_bufs * (L.KP + L.ZP) * L.ZP);
-  L.slice_len = nc > 0 ? ((L.KP + L.ZP) * L.ZP + nc - 1) / nc + 4 : 0;
-  L.slice = take(2 * (size_t)L.slice_len);
-  L.P = take((size_t)L.KP * L.ZP);
-  L.Gm = take((size_t)zmax * (zmax + 1));
-  L.T = take((size_t)L.ZP * L.ZP);
-  L.R = take((size_t)zmax * zmax);
-  L.misc = take(256);
-  L.Zc = take((size_t)L.RP * L.ZP);
-  L.Zn = take((size_t)L.RP * L.ZP);
-  L.Qc = take((size_t)L.RP * L.KP);
-  // split partial products: at most 512 tiles of 16 sums (tn_split)
-  L.tmp = take(imin(8192, 8 * (size_t)L.ZP * imax(L.KP, L.ZP)));
-  L.total = o;
-  return L;
-}
 
 // Y[i][j] = scale * sum_{t < kk} X[i][t] M[t][j] (+ Y0[i][j]) for i < rows,
 // j < bp (rows, kk, bp and the row strides multiples of 4).  A warp takes
@@ -568,13 +535,6 @@ bool kc_schedulable(int nc, size_t smem) {
   return ok;
 }
 
-// Grid form: one CTA per SM at most (every CTA of the cooperative launch
-// resident), at least 16 rows each.
-struct KgConfig {
-  int nr = 0, rows = 0, E = 0;
-  size_t smem = 0;
-};
-
 int kg_device_ctas() {
   static std::mutex mu;
   static std::map<int, int> cache;
@@ -592,46 +552,27 @@ int kg_device_ctas() {
   return sms;
 }
 
-bool kg_config(int64_t m, int kqmax, int zmax, KgConfig* cfg) {
-  if (m < 1 || zmax < 1 || zmax > 64 || kqmax > 256) return false;
-  const int maxr = kg_device_ctas();
-  if (maxr < 1) return false;
-  const int64_t nr0 = imin((int64_t)maxr, imax((int64_t)1, ceil_div(m, 16)));
-  const int64_t rows = ceil_div(m, nr0);
-  const KcLayout L = kc_layout(kqmax, zmax, (int)rows, 0);
-  const size_t smem = L.total * sizeof(float);
-  if (smem > (size_t)KC_SMEM_MAX) return false;
-  cfg->rows = (int)rows;
-  cfg->nr = (int)ceil_div(m, rows);
-  cfg->E = (L.KP + L.ZP) * L.ZP;
-  cfg->smem = smem;
-  return true;
-}
-
 }  // namespace
 
-bool orth_grid_rs_ok(int64_t m, int kq0, int zc, int c) {
-  KgConfig cfg;
-  return c >= 1 && c <= zc && kg_config(m, kq0 + c, zc, &cfg);
-}
-
-size_t orth_grid_rs_scratch_floats(int64_t m, int kq0, int zc) {
-  KgConfig cfg;
-  if (!kg_config(m, kq0 + zc, zc, &cfg)) return 0;
-  return 4 + 2 * (size_t)cfg.nr * cfg.E + 2 * (size_t)cfg.E;
+OrthGridLimits orth_grid_limits() {
+  OrthGridLimits l;
+  l.ctas = kg_device_ctas();
+  l.smem = KC_SMEM_MAX;
+  return l;
 }
 
 cudaError_t launch_orth_grid_rs(const float* Y, int64_t ldy, int zc, int64_t m, int c, int kq0, float* Q,
-                                int64_t ldq, float* Xg, int xld, uint64_t seed, float* scratch, int* status,
-                                cudaStream_t st) {
+                                int64_t ldq, float* Xg, int xld, uint64_t seed, float* scratch,
+                                size_t scratch_floats, int* status, cudaStream_t st) {
   if (c < 1 || c > zc || (Xg && xld < pad4(c)) || !scratch) return cudaErrorInvalidValue;
   OrthRsArgs a = {};
   a.Y = Y; a.ldy = ldy; a.Q = Q; a.ldq = ldq; a.Xg = Xg; a.xld = xld; a.m = m;
   a.kq0 = kq0; a.zc0 = zc; a.c = c; a.status = status; a.seed = seed;
   a.kqmax = kq0 + c;
   a.zmax = zc;
-  KgConfig cfg;
-  if (!kg_config(m, a.kqmax, zc, &cfg)) return cudaErrorInvalidValue;
+  OrthGridShape cfg;
+  if (!orth_grid_shape(m, a.kqmax, zc, orth_grid_limits(), &cfg)) return cudaErrorInvalidValue;
+  if (cfg.scratch_floats() > scratch_floats) return cudaErrorInvalidValue;   // the shares would run past it
   a.rows = cfg.rows;
   a.eslot = cfg.E;
   a.gbar = reinterpret_cast<unsigned*>(scratch);

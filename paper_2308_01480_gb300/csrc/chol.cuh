@@ -169,11 +169,15 @@ __device__ __forceinline__ void inv_warp(CholShared<W>& sh, int b) {
   }
 }
 
-// One per kernel and width.
+// One per kernel, shared by both widths: no call is inside another.
+__device__ __forceinline__ float* chol_shared_words() {
+  static_assert(sizeof(CholShared<16>) <= sizeof(CholShared<32>), "the wide form is the larger");
+  __shared__ __align__(16) float words[sizeof(CholShared<32>) / sizeof(float)];
+  return words;
+}
 template <int W>
 __device__ __forceinline__ CholShared<W>& chol_shared() {
-  __shared__ __align__(16) CholShared<W> sh;
-  return sh;
+  return *reinterpret_cast<CholShared<W>*>(chol_shared_words());
 }
 
 // Out of line (one copy per kernel, its own register allocation).

@@ -123,6 +123,13 @@ template <typename Kernel>
 inline cudaError_t raise_smem_limit(Kernel kernel) {
   return raise_smem_limit_ptr(reinterpret_cast<const void*>(kernel));
 }
+// That limit in bytes (0 without a device), for the rules that decide whether
+// a shape fits the kernel.
+size_t dynamic_smem_limit_ptr(const void* kernel);
+template <typename Kernel>
+inline size_t dynamic_smem_limit(Kernel kernel) {
+  return dynamic_smem_limit_ptr(reinterpret_cast<const void*>(kernel));
+}
 
 __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 __host__ __device__ inline int64_t imin(int64_t a, int64_t b) { return a < b ? a : b; }

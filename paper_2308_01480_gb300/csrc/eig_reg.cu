@@ -978,7 +978,7 @@ static int er_kt(int k) { return (k + 31) / 32; }
 bool eig_reg_ok(int k, int r) {
   if (k < 1 || r < 1 || r > 32 || r > k || k > 32 * ER_KTMAX) return false;
   // dynamic shared memory plus the kernel's static arrays (the Cholesky's
-  // rows, 8.5 KB + 2.2 KB) within the 227 KB a CTA may use
+  // 8,448 bytes, 12 KB reserved) within the 227 KB a CTA may use
   return er_layout(32 * er_kt(k), k, r).total * 4 + 12 * 1024 <= 227 * 1024;
 }
 

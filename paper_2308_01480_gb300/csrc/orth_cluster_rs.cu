@@ -39,7 +39,6 @@ namespace {
 
 constexpr int KC_THREADS = 512;
 constexpr int KC_MAX_ROWS = 64;
-constexpr int KC_SMEM_MAX = 218 * 1024;
 
 struct OrthRsArgs {
   const float* Y;       // the block, m x zc0, row stride ldy
@@ -496,7 +495,7 @@ bool kc_config(int64_t m, int kqmax, int zmax, KcConfig* cfg) {
   if (rows > KC_MAX_ROWS) return false;
   const KcLayout L = kc_layout(kqmax, zmax, (int)rows, nc);
   const size_t smem = L.total * sizeof(float);
-  if (smem > (size_t)KC_SMEM_MAX) return false;
+  if (smem > dynamic_smem_limit(k_orth_cluster_rs)) return false;
   cfg->nc = nc;
   cfg->rows = (int)rows;
   cfg->smem = smem;
@@ -557,7 +556,7 @@ int kg_device_ctas() {
 OrthGridLimits orth_grid_limits() {
   OrthGridLimits l;
   l.ctas = kg_device_ctas();
-  l.smem = KC_SMEM_MAX;
+  if (l.ctas > 0) l.smem = dynamic_smem_limit(k_orth_grid_rs);   // beside the kernel's static arrays
   return l;
 }
 

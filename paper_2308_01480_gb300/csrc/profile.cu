@@ -55,24 +55,47 @@ ProfScope::~ProfScope() {
   g_recs.push_back({fam_, a_, b_});
 }
 
-cudaError_t raise_smem_limit_ptr(const void* kernel) {
+namespace {
+
+// Per device and kernel: the largest dynamic shared memory of a CTA (0 when
+// it cannot be asked) and the outcome of raising the kernel's limit to it.
+struct SmemLimit {
+  size_t bytes = 0;
+  cudaError_t query = cudaSuccess, raise = cudaSuccess;
+  bool raised = false;
+};
+
+SmemLimit smem_limit_entry(const void* kernel, bool raise) {
   static std::mutex mu;
-  static std::map<std::pair<int, const void*>, cudaError_t> done;
+  static std::map<std::pair<int, const void*>, SmemLimit> done;
+  SmemLimit l;
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
+  l.query = l.raise = cudaGetDevice(&dev);
+  if (l.query != cudaSuccess) return l;
   std::lock_guard<std::mutex> lk(mu);
   auto it = done.find({dev, kernel});
-  if (it != done.end()) return it->second;
-  cudaFuncAttributes fa;
-  int optin = 0;
-  e = cudaFuncGetAttributes(&fa, kernel);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-  done[{dev, kernel}] = e;
-  return e;
+  if (it == done.end()) {
+    cudaFuncAttributes fa;
+    int optin = 0;
+    l.query = cudaFuncGetAttributes(&fa, kernel);
+    if (l.query == cudaSuccess)
+      l.query = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (l.query == cudaSuccess && optin > (int)fa.sharedSizeBytes) l.bytes = (size_t)optin - fa.sharedSizeBytes;
+    if (l.query != cudaSuccess) cudaGetLastError();   // reported through the entry
+    l.raise = l.query;
+    it = done.insert({{dev, kernel}, l}).first;
+  }
+  if (raise && !it->second.raised && it->second.query == cudaSuccess) {
+    it->second.raise = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)it->second.bytes);
+    it->second.raised = true;
+  }
+  return it->second;
 }
+
+}  // namespace
+
+cudaError_t raise_smem_limit_ptr(const void* kernel) { return smem_limit_entry(kernel, true).raise; }
+size_t dynamic_smem_limit_ptr(const void* kernel) { return smem_limit_entry(kernel, false).bytes; }
 
 }  // namespace ttr
 

@@ -1,6 +1,6 @@
-"""Tall wide modes whose first Krylov blocks take the grid form of the block
-orthonormalisation and whose last does not, in a workspace of exactly the
-queried size with guard bytes behind it, against the float64 oracle."""
+"""The grid form of the block orthonormalisation at the edges of its launch
+rules, in a workspace of exactly the queried size with guard bytes behind it,
+against the float64 oracle."""
 import numpy as np
 import pytest
 import torch
@@ -10,8 +10,7 @@ pytestmark = pytest.mark.gpu
 GUARD = 8 << 20
 
 
-@pytest.mark.parametrize("dims,r,p,q", [((250, 250, 250), 45, 10, 2), ((9000, 300), 40, 10, 3), ((9000, 300), 56, 8, 1)])
-def test_mixed_routes_stay_in_the_workspace(dims, r, p, q):
+def _check(dims, r, p, q):
     import oracle
     import paper_2308_01480_gb300 as tt
     rng = np.random.default_rng(sum(dims))
@@ -32,3 +31,20 @@ def test_mixed_routes_stay_in_the_workspace(dims, r, p, q):
     ref = oracle.tt_rbki(A, ranks, p, q, seed=3)
     # the repository's FP32 criterion
     assert oracle.tt_distance([c.cpu().double().numpy() for c in cores], ref) <= 1e-4
+
+
+@pytest.mark.parametrize("dims,r,p,q", [((250, 250, 250), 45, 10, 2), ((9000, 300), 40, 10, 3), ((9000, 300), 56, 8, 1)])
+def test_mixed_routes_stay_in_the_workspace(dims, r, p, q):
+    """The first blocks take the grid form, the last does not."""
+    _check(dims, r, p, q)
+
+
+@pytest.mark.parametrize("m,r,p,q", [(22800, 20, 10, 4),    # 219,552 bytes of dynamic shared memory in the last block
+                                     (44000, 10, 10, 4),    # 219,792
+                                     (12000, 40, 10, 2),    # 220,784
+                                     (43200, 9, 8, 5),      # 221,920
+                                     (10300, 38, 10, 3)])   # 222,912: more than a CTA has beside the static arrays
+def test_blocks_near_the_shared_memory_limit(m, r, p, q):
+    """Layouts just inside and just outside what a CTA can have: either the
+    grid form runs or another route does, none is refused at its launch."""
+    _check((m, (r + p) * (q + 1) + 10), r, p, q)

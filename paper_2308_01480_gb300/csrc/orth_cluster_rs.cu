@@ -49,6 +49,7 @@ struct OrthRsArgs {
   int xld;
   int64_t m;
   int rows;             // rows per CTA
+  bool tight;           // the smaller shared-memory layout
   int kq0;              // basis columns already in Q
   int zc0;              // columns of Y
   int c;                // columns kept
@@ -132,13 +133,15 @@ __device__ void nn_any(const float* X, int ldx, int kk, const float* M, int ldm,
 
 // out[t][j] = sum_{i < rows} A[i][t] B[i][j] (t < ta, j < bp, multiples of 4)
 // with the rows split over KS groups of threads when there are few output
-// tiles; the KS partial tiles (in tmp) are summed in group order.  Ends
+// tiles; the KS partial tiles (in tmp, of tmp_len floats) are summed in group
+// order.  Ends
 // with a __syncthreads().
 __device__ void tn_split(const float* A, int lda, int ta, const float* B, int ldb, int bp, int rows, float* out,
-                         int ldo, float* tmp) {
+                         int ldo, float* tmp, int tmp_len) {
   const int tt = ta >> 2, tj = bp >> 2, tiles = tt * tj;
-  const int KS = 4 * tiles <= (int)blockDim.x ? imin(8, (int)blockDim.x / tiles) : 1;
-  if (KS == 1) {
+  const int KS =
+      4 * tiles <= (int)blockDim.x ? imin(imin(8, (int)blockDim.x / tiles), tmp_len / (16 * tiles)) : 1;
+  if (KS <= 1) {
     tn_tile(A, lda, ta, B, ldb, bp, rows, out, ldo);
     __syncthreads();
     return;
@@ -334,8 +337,8 @@ __device__ __forceinline__ void orth_rs_body(const OrthRsArgs& a, Comm& comm, fl
       __syncthreads();
       auto reduce = [&](bool qz, bool zz) {
         float* mine = share0 + (size_t)(L.share_bufs == 2 ? (phase & 1) : 0) * (KP + ZP) * ZP;
-        if (qz) tn_split(Qc, KP, kp, Zc, ZP, bz, RP, mine, bz, tmp);
-        if (zz) tn_split(Zc, ZP, bz, Zc, ZP, bz, RP, mine + kp * bz, bz, tmp);
+        if (qz) tn_split(Qc, KP, kp, Zc, ZP, bz, RP, mine, bz, tmp, L.tmp_len);
+        if (zz) tn_split(Zc, ZP, bz, Zc, ZP, bz, RP, mine + kp * bz, bz, tmp, L.tmp_len);
         __syncthreads();
         const int e0 = qz ? 0 : kp * bz, e1 = zz ? E : kp * bz;
         auto put = [&](int e, float s) {
@@ -457,7 +460,7 @@ __global__ void __launch_bounds__(KC_THREADS, 1) k_orth_cluster_rs(const __grid_
   extern __shared__ __align__(16) float sm[];
   __shared__ unsigned long long badmask;
   ClusterComm comm{cg::this_cluster(), nullptr, 0};
-  const KcLayout L = kc_layout(a.kqmax, a.zmax, a.rows, comm.nranks());
+  const KcLayout L = kc_layout(a.kqmax, a.zmax, a.rows, comm.nranks(), a.tight);
   comm.slices = sm + L.slice;
   comm.slice_len = L.slice_len;
   orth_rs_body(a, comm, sm, L, badmask);
@@ -473,7 +476,7 @@ __global__ void __launch_bounds__(KC_THREADS, 1) k_orth_grid_rs(const __grid_con
   if (threadIdx.x == 0) dead = 0;
   __syncthreads();
   GridComm comm{(int)gridDim.x, (int)blockIdx.x, a.gparts, a.gsums, a.eslot, a.gbar, a.status, &dead, gtmp};
-  const KcLayout L = kc_layout(a.kqmax, a.zmax, a.rows, 0);
+  const KcLayout L = kc_layout(a.kqmax, a.zmax, a.rows, 0, a.tight);
   orth_rs_body(a, comm, sm, L, badmask);
 }
 
@@ -484,6 +487,7 @@ namespace {
 
 struct KcConfig {
   int nc = 0, rows = 0;
+  bool tight = false;
   size_t smem = 0;
 };
 
@@ -493,9 +497,11 @@ bool kc_config(int64_t m, int kqmax, int zmax, KcConfig* cfg) {
   while (nc < 16 && ceil_div(m, nc) > KC_MAX_ROWS) nc *= 2;
   const int64_t rows = ceil_div(m, nc);
   if (rows > KC_MAX_ROWS) return false;
-  const KcLayout L = kc_layout(kqmax, zmax, (int)rows, nc);
-  const size_t smem = L.total * sizeof(float);
-  if (smem > dynamic_smem_limit(k_orth_cluster_rs)) return false;
+  const size_t limit = dynamic_smem_limit(k_orth_cluster_rs);
+  size_t smem = kc_layout(kqmax, zmax, (int)rows, nc, false).total * sizeof(float);
+  cfg->tight = smem > limit;
+  if (cfg->tight) smem = kc_layout(kqmax, zmax, (int)rows, nc, true).total * sizeof(float);
+  if (smem > limit) return false;
   cfg->nc = nc;
   cfg->rows = (int)rows;
   cfg->smem = smem;
@@ -573,6 +579,7 @@ cudaError_t launch_orth_grid_rs(const float* Y, int64_t ldy, int zc, int64_t m, 
   if (!orth_grid_shape(m, a.kqmax, zc, orth_grid_limits(), &cfg)) return cudaErrorInvalidValue;
   if (cfg.scratch_floats() > scratch_floats) return cudaErrorInvalidValue;   // the shares would run past it
   a.rows = cfg.rows;
+  a.tight = cfg.tight;
   a.eslot = cfg.E;
   a.gbar = reinterpret_cast<unsigned*>(scratch);
   a.gparts = scratch + 4;
@@ -615,6 +622,7 @@ cudaError_t launch_orth_cluster_rs(const float* Y, int64_t ldy, int zc, int64_t 
   if (!kc_config(m, a.kqmax, zc, &cfg)) return cudaErrorInvalidValue;
   if (!kc_schedulable(cfg.nc, cfg.smem)) return cudaErrorNotSupported;
   a.rows = cfg.rows;
+  a.tight = cfg.tight;
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(cfg.nc);
   lc.blockDim = dim3(KC_THREADS);

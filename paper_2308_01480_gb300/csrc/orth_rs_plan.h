@@ -26,13 +26,17 @@ namespace ttr {
 struct KcLayout {
   int KP, ZP, RP;
   size_t share, slice, P, Gm, T, R, misc, Zc, Zn, Qc, tmp, total;
+  int tmp_len;          // floats of tmp
   int slice_len;
   int share_bufs;       // 2 for a cluster (other ranks read the shares), 1 for the grid form
 };
 
 // nc: cluster size; nc = 0 for the grid form (shares and sums in global
-// memory, no slice buffers).
-TTR_HD inline KcLayout kc_layout(int kqmax, int zmax, int rows, int nc) {
+// memory, no slice buffers).  tight: the split partial products keep room for
+// the block's own Gram only, and Q^T Z is split less or not at all; for
+// blocks that fit no other way (44,000 x 20 against 80 columns: 200 KB instead
+// of 220 KB a CTA; the next route takes several launches).
+TTR_HD inline KcLayout kc_layout(int kqmax, int zmax, int rows, int nc, bool tight) {
   KcLayout L;
   L.KP = (kqmax + 3) & ~3;
   L.ZP = (zmax + 3) & ~3;
@@ -52,8 +56,9 @@ TTR_HD inline KcLayout kc_layout(int kqmax, int zmax, int rows, int nc) {
   L.Zn = take((size_t)L.RP * L.ZP);
   L.Qc = take((size_t)L.RP * L.KP);
   // split partial products: at most 512 tiles of 16 sums (tn_split)
-  const size_t split = 8 * (size_t)L.ZP * (L.KP > L.ZP ? L.KP : L.ZP);
-  L.tmp = take(split < 8192 ? split : 8192);
+  const size_t split = 8 * (size_t)L.ZP * (!tight && L.KP > L.ZP ? L.KP : L.ZP);
+  L.tmp_len = (int)(split < 8192 ? split : 8192);
+  L.tmp = take((size_t)L.tmp_len);
   L.total = o;
   return L;
 }
@@ -68,6 +73,7 @@ struct OrthGridLimits {
 // Shape of one grid-form call: nr CTAs of `rows` rows, shares of E floats.
 struct OrthGridShape {
   int nr = 0, rows = 0, E = 0;
+  bool tight = false;
   size_t smem = 0;
   // barrier words, two buffers of nr shares, two of their sums
   size_t scratch_floats() const { return 4 + 2 * (size_t)nr * E + 2 * (size_t)E; }
@@ -81,7 +87,9 @@ inline bool orth_grid_shape(int64_t m, int kqmax, int zmax, const OrthGridLimits
   if (nr0 > lim.ctas) nr0 = lim.ctas;
   const int64_t rows = (m + nr0 - 1) / nr0;
   if (rows > (1 << 20)) return false;          // far beyond shared memory; keeps the layout's ints in range
-  const KcLayout L = kc_layout(kqmax, zmax, (int)rows, 0);
+  KcLayout L = kc_layout(kqmax, zmax, (int)rows, 0, false);
+  s->tight = L.total * sizeof(float) > lim.smem;
+  if (s->tight) L = kc_layout(kqmax, zmax, (int)rows, 0, true);
   const size_t smem = L.total * sizeof(float);
   if (smem > lim.smem) return false;
   s->rows = (int)rows;

@@ -48,3 +48,9 @@ def test_blocks_near_the_shared_memory_limit(m, r, p, q):
     """Layouts just inside and just outside what a CTA can have: either the
     grid form runs or another route does, none is refused at its launch."""
     _check((m, (r + p) * (q + 1) + 10), r, p, q)
+
+
+@pytest.mark.parametrize("m,r,p,q", [(44394, 10, 8, 5), (40417, 11, 10, 4), (45946, 16, 10, 2)])
+def test_blocks_in_the_tight_layout(m, r, p, q):
+    """Layouts that leave no room to split Q^T Z over groups of threads."""
+    _check((m, (r + p) * (q + 1) + 10), r, p, q)

@@ -110,3 +110,12 @@ def test_restarted_calls_and_no_device(plan):
     scratch, need = _mode(plan, 12000, 60, 3, restarts=1)
     assert len(need) == 2 and scratch == max(need) > 0
     assert _mode(plan, 12000, 60, 3, ctas=0) == (0, [-1] * 4)
+
+
+@pytest.mark.parametrize("m,b,q,full", [(44394, 18, 5, 232176), (40417, 21, 4, 230000), (45946, 26, 2, 228880)])
+def test_blocks_that_fit_only_the_tight_layout_keep_the_grid_form(plan, m, b, q, full):
+    """Layouts whose split partial products, sized for Q^T Z as well, take the
+    last block past the 221,920 bytes of a CTA."""
+    assert full > 221920
+    scratch, need = _mode(plan, m, b, q, smem=221920)
+    assert min(need) > 0 and scratch == max(need)

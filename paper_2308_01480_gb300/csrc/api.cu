@@ -235,8 +235,11 @@ tt_status build_plan(const int64_t* dims, int d, const int64_t* ranks, int p, in
     } else {
       maxS = std::max(maxS, (size_t)(M.b * M.n));
       maxPart = std::max(maxPart, (size_t)ttr::simt_cs_partials(M.m, M.n, M.b));
+      // a power runs at its block's width, and a narrower one may have more
+      // CTAs (two an SM where b columns leave room for one), so more partials
       if (M.fused_ga)
-        maxPart = std::max(maxPart, (size_t)ttr::simt_ga_partials(M.m, M.n, M.b));
+        for (const int c : M.blocks)
+          maxPart = std::max(maxPart, (size_t)ttr::simt_ga_partials(M.m, M.n, c));
       else
         maxT = std::max(maxT, (size_t)(M.b * M.n));
       maxY = std::max(maxY, (size_t)(M.m * M.b));

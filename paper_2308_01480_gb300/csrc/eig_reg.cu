@@ -27,6 +27,7 @@
 #include "cluster_la.cuh"
 #include "common.cuh"
 #include "kernels.h"
+#include "sturm.cuh"
 
 namespace ttr {
 
@@ -65,75 +66,6 @@ __device__ __forceinline__ int warp_min_i(int v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
-}
-
-// Number of eigenvalues of the scaled T below x: sign changes of the leading
-// principal minors p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (Givens 1953),
-// de[i] = (d_i, e_{i-1}^2), |T| < 2.  One multiply-add a row is on the chain
-// (the ratios p_i / p_{i-1} would put a reciprocal and a comparison there);
-// every four rows the pair is rescaled by a power of two.  Rows past the last
-// are padded by (16, 0), which changes no sign, up to 1 + 4 groups rows.
-// k = 150: 75 to 100 cycles a row as ratios, about 55 (two counts a warp).
-struct SturmPair {
-  float p0, p1;
-  unsigned m;        // signs of the last p's, newest in bit 0
-  int c;
-  __device__ __forceinline__ void start(float2 t, float x) {
-    p0 = 1.f;
-    p1 = t.x - x;
-    m = __float_as_uint(p1) >> 31;
-    c = (int)m;
-  }
-  __device__ __forceinline__ void step(float d, float e2, float x) {
-    const float pn = fmaf(d - x, p1, -(e2 * p0));
-    m = __funnelshift_l(__float_as_uint(pn), m, 1);
-    p0 = p1;
-    p1 = pn;
-  }
-  // after every four steps
-  __device__ __forceinline__ void settle() {
-    c += __popc((m ^ (m >> 1)) & 15u);
-    const float f0 = fmaxf(fabsf(p0), fabsf(p1));
-    const float f = __uint_as_float(0x7f000000u - (__float_as_uint(f0) & 0x7f800000u));
-    p0 *= f;
-    p1 = (f0 == 0.f) ? 1.f : p1 * f;     // both zero: the rows decouple here
-  }
-};
-
-// Rows 1 .. 4 groups are read as pairs: de + 1 is 16-byte aligned.
-__device__ __forceinline__ int sturm(const float2* de, int groups, float x) {
-  SturmPair s;
-  s.start(de[0], x);
-  const float4* q = reinterpret_cast<const float4*>(de + 1);
-#pragma unroll 2
-  for (int g = 0; g < groups; ++g) {
-    const float4 a = q[2 * g], b = q[2 * g + 1];
-    s.step(a.x, a.y, x);
-    s.step(a.z, a.w, x);
-    s.step(b.x, b.y, x);
-    s.step(b.z, b.w, x);
-    s.settle();
-  }
-  return s.c;
-}
-
-// Two counts (at x0 and x1) in one pass, so that the two chains overlap.
-__device__ __forceinline__ void sturm2(const float2* de, int groups, float x0, float x1, int& c0, int& c1) {
-  SturmPair s0, s1;
-  s0.start(de[0], x0);
-  s1.start(de[0], x1);
-  const float4* q = reinterpret_cast<const float4*>(de + 1);
-  for (int g = 0; g < groups; ++g) {
-    const float4 a = q[2 * g], b = q[2 * g + 1];
-    s0.step(a.x, a.y, x0); s1.step(a.x, a.y, x1);
-    s0.step(a.z, a.w, x0); s1.step(a.z, a.w, x1);
-    s0.step(b.x, b.y, x0); s1.step(b.x, b.y, x1);
-    s0.step(b.z, b.w, x0); s1.step(b.z, b.w, x1);
-    s0.settle();
-    s1.settle();
-  }
-  c0 = s0.c;
-  c1 = s1.c;
 }
 
 // Pivoted LU of T - lam I, one thread per vector: row i of w holds
@@ -605,8 +537,7 @@ __global__ void __launch_bounds__(512, 1) k_eig_vectors(const float* __restrict_
   const float up = __uint_as_float(0x7f000000u - ex), down = __uint_as_float(ex);
   const int groups4 = (k + 2) / 4;        // 1 + 4 groups4 >= k rows
   for (int i = tid; i < 1 + 4 * groups4; i += NT) {
-    const float es = (i > 0 && i < k) ? e[i - 1] * up : 0.f;
-    de[i] = (i < k) ? make_float2(d[i] * up, es * es) : make_float2(16.f, 0.f);
+    de[i] = (i < k) ? sturm_row(d[i] * up, i > 0 ? e[i - 1] * up : 0.f) : sturm_row(16.f, 0.f);
   }
   __syncthreads();
   const float pad = 4.f * FLT_EPSILON;

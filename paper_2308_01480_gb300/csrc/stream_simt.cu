@@ -240,7 +240,7 @@ cudaError_t launch_reduce_partials_grouped(const float* P, int per, int groups, 
 
 namespace {
 
-// Rows of a cs tile: the shortest of 32, 48 and 64 that needs no more tiles.
+// Rows of a cs tile: the shortest of 32, 48 and 64 that takes all rows, else 64.
 int cs_tile_rows(int64_t m) { return m <= 32 ? 32 : m <= 48 ? 48 : 64; }
 
 // Two CTAs an SM in all, a split at least 256 columns.
@@ -258,8 +258,9 @@ cudaError_t cs_launch(const TIn* C, int64_t m, int64_t n, const float* S, int64_
     const cudaError_t e = raise_smem_limit(k_cs<Sh, TIn>);
     if (e != cudaSuccess) return e;
   }
+  // vector loads end with the row only where n is a multiple of four, however S is spaced
   k_cs<Sh, TIn><<<dim3((unsigned)ceil_div(m, Sh::BM), (unsigned)splits), 256, smem, st>>>(
-      C, m, n, S, lds, b, P, per, simt::rows_aligned4(C, n), simt::rows_aligned4(S, lds));
+      C, m, n, S, lds, b, P, per, simt::rows_aligned4(C, n), n % 4 == 0 && simt::rows_aligned4(S, lds));
   return cudaGetLastError();
 }
 

@@ -307,19 +307,40 @@ int64_t simt_cs_partials(int64_t m, int64_t n, int b) { return cs_splits(m, n) *
 // ---------------------------------------------------------------- gram
 namespace {
 
-// Tile edge: 48 or 64, whichever pads the rows to less (64 on a tie); one tile
-// of 16 or 32 for the shortest.
-int gram_tile(int64_t m) {
-  if (m <= 32) return m <= 16 ? 16 : 32;
-  return ceil_div(m, 48) * 48 < ceil_div(m, 64) * 64 ? 48 : 64;
-}
+// Tile edge, tiles of the upper triangle and splits of the columns.
+struct GramPlan {
+  int edge, tiles, splits;
+};
 
-// Tiles of the upper triangle and splits of the columns: two CTAs an SM, a
-// split at least 256 columns.
-void gram_plan(int64_t m, int64_t n, int* tiles, int* splits) {
-  const int nT = (int)ceil_div(m, gram_tile(m));
-  *tiles = nT * (nT + 1) / 2;
-  *splits = (int)imax(1, imin(2 * 152 / *tiles, ceil_div(n, 256)));
+// One tile of 16 or 32 for the shortest; else of 48 and 64 the edge, and of
+// the splits that give every SM one CTA or two, those with the least time by
+//   (chunks of a CTA + 1/2) x (1.85 per two CTAs an SM holds, 1 for one alone)
+// plus one where more than eight partials are left to add, with a chunk of a
+// 64-row tile 1.6 times a 48-row one (the ratios measured at 200 to 1,000
+// rows).  The splits go down to one chunk, since a short Gram is one chain of
+// chunks.  A fixed minimum of 256 columns a split and the edge by padding alone
+// gave 700 columns of 39 rows three CTAs (9.5 us, so 5.7) and 800 x 8,000
+// one CTA of 48 rows an SM (276 us, 176 as 64-row tiles in three splits).
+GramPlan gram_plan(int64_t m, int64_t n) {
+  const int64_t chunks = ceil_div(n, 64);
+  GramPlan best = {};
+  double least = 0.;
+  for (const int edge : {16, 32, 48, 64}) {
+    if (m <= 32 ? edge != (m <= 16 ? 16 : 32) : edge < 48) continue;
+    const int64_t nT = ceil_div(m, edge), tiles = nT * (nT + 1) / 2;
+    for (const int64_t ctas : {152, 304}) {
+      int64_t splits = imax(1, imin(ctas / tiles, chunks));
+      const int64_t per = ceil_div(chunks, splits);
+      splits = ceil_div(chunks, per);
+      const int64_t held = ceil_div(tiles * splits, 152);     // CTAs of the fullest SM
+      const double t = (per + 0.5) * ((held / 2) * 1.85 + held % 2) * (edge == 64 ? 1.6 : 1.) + (splits > 8);
+      if (best.edge == 0 || t < least) {
+        least = t;
+        best = {edge, (int)tiles, (int)splits};
+      }
+    }
+  }
+  return best;
 }
 
 template <class Sh, typename TIn>
@@ -346,23 +367,20 @@ cudaError_t gram_launch(const TIn* C, int64_t m, int64_t n, int tiles, int split
 template <typename TIn>
 cudaError_t simt_gram(const TIn* C, int64_t m, int64_t n, float* partials, float* out, cudaStream_t st,
                       const char* family) {
-  int tiles, splits;
-  gram_plan(m, n, &tiles, &splits);
+  const GramPlan p = gram_plan(m, n);
   ProfScope prof(family, st, (double)m * n * sizeof(TIn), 2.0 * m * m * n);
   note_launch(family);
-  switch (gram_tile(m)) {
-    case 16: return gram_launch<simt::NtShape<2, 8, 2>>(C, m, n, tiles, splits, partials, out, st);
-    case 32: return gram_launch<simt::NtShape<4, 8, 4>>(C, m, n, tiles, splits, partials, out, st);
-    case 48: return gram_launch<simt::NtShape<6, 6, 8>>(C, m, n, tiles, splits, partials, out, st);
-    default: return gram_launch<simt::NtShape<8, 4, 16>>(C, m, n, tiles, splits, partials, out, st);
+  switch (p.edge) {
+    case 16: return gram_launch<simt::NtShape<2, 8, 2>>(C, m, n, p.tiles, p.splits, partials, out, st);
+    case 32: return gram_launch<simt::NtShape<4, 8, 4>>(C, m, n, p.tiles, p.splits, partials, out, st);
+    case 48: return gram_launch<simt::NtShape<6, 6, 8>>(C, m, n, p.tiles, p.splits, partials, out, st);
+    default: return gram_launch<simt::NtShape<8, 4, 16>>(C, m, n, p.tiles, p.splits, partials, out, st);
   }
 }
 
 int64_t simt_gram_partials(int64_t m, int64_t n) {
-  int tiles, splits;
-  gram_plan(m, n, &tiles, &splits);
-  const int64_t t = gram_tile(m);
-  return (int64_t)tiles * splits * t * t;
+  const GramPlan p = gram_plan(m, n);
+  return (int64_t)p.tiles * p.splits * p.edge * p.edge;
 }
 
 // Explicit instantiations.

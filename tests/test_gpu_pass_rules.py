@@ -1,0 +1,31 @@
+"""The CUDA-core passes on both sides of their launch rules: the Gram's tile
+edge and splits; against a float64 recomputation."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+GRAM = [(m, n) for m in (1, 16, 17, 32, 33, 64, 100, 240, 400) for n in (1, 64, 65, 700, 2001)] + [(800, 1601), (1000, 300), (39, 20011)]
+
+
+def _case(m, n, b, dtype):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m * 7 + n + b)
+    C = torch.randn(m, n, generator=g, device="cuda").to(getattr(torch, dtype))
+    return C, torch.randn(m, b, generator=g, device="cuda")
+
+
+def _check(got, ref, bound):
+    # FP32 sums: the repository's 1e-5 of the largest absolute-value bound
+    assert float((got.double() - ref).abs().max()) <= 1e-5 * float(bound.max())
+
+
+@pytest.mark.parametrize("dtype", ["float32", "bfloat16"])
+def test_gram_rules(dtype):
+    import paper_2308_01480_gb300 as tt
+    for m, n in GRAM:
+        n += 1 if dtype == "bfloat16" and n % 8 == 0 else 0
+        C, _ = _case(m, n, 1, dtype)
+        G = tt.tt_pass(tt.TT_PASS_GRAM, C)
+        _check(G, C.double() @ C.double().T, C.double().abs() @ C.double().abs().T)
+        assert torch.equal(G, G.T)

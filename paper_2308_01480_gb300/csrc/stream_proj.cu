@@ -4,16 +4,19 @@
 //
 // Every column of C is one column of S, so a thread keeps four whole
 // columns (TC sums of each) in registers and reads C straight from global
-// memory, coalesced along the row: C needs no shared memory and no barrier.  X is the small operand: chunks of 16 rows are double-buffered in
-// shared memory by each row group for itself (a barrier over the CTA per
-// chunk held up the others) and read as broadcasts, one 16-byte load for 16
-// multiply-adds, two to an instruction.  The next rows of C (16 to 32 elements a thread) are in
-// flight while the current ones are multiplied.
+// memory, coalesced along the row: C needs no shared memory and no barrier.
+// X is the small operand: chunks of 16 rows are double-buffered in shared
+// memory by each row group for itself (a barrier over the CTA per chunk held
+// up the others) and read as broadcasts, one 16-byte load for 16
+// multiply-adds, two to an instruction.  The next rows of C (16 to 32 elements
+// a thread) are in flight while the current ones are multiplied.
 // The eight warps of a CTA split into CG groups of output rows (b > 20), RG
 // groups of rows of C (few columns: the groups' sums are added in order) and
 // the rest over columns; when even that leaves the chip idle (n below
 // 128 x 152 columns), the rows are also split over the grid and a second
-// kernel adds the partials in split order.
+// kernel adds the partials in split order.  Few rows of wide or short
+// unfoldings take tiles of 64 columns with both operands in shared memory
+// (k_proj_tile).
 // Measured (FP32, us; before: 16 x 16 threads with both operands staged in
 // shared memory and no split over rows unless n <= 512): 7680 x 2048 at
 // b = 20 404 -> 31, 800 x 64,000 at b = 20 190 -> 106, 45 x 4,100,625 at
@@ -29,11 +32,6 @@ namespace {
 
 constexpr int PJ_RK = 16;   // rows of X per shared-memory chunk of a row group
 constexpr int PJ_NC = 4;    // columns of C per thread
-
-__device__ __forceinline__ void cp_async16z(float* dst, const float* src, bool ok) {
-  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
-}
 
 // VEC: every row of C (and of S) starts aligned to four elements, and the
 // thread's columns are neighbours; otherwise they are 32 apart.  x16: rows
@@ -215,48 +213,168 @@ __global__ void k_sum_splits(const float* __restrict__ P, int splits, int b, int
   }
 }
 
-template <typename TIn, typename TOut, int TC>
+// The form for at most 256 rows of wide or short unfoldings: 64 columns x
+// 16 VB rows of S a CTA, both operands staged in shared memory 32 rows at a
+// time (proj_tile says where).  Three or four CTAs an SM leave the registers for every
+// load of a chunk to be in flight (at 32 they took turns: 64 x 16,384 at
+// b = 20 8.1 us, 6.1 so).
+template <typename TIn, typename TOut, int VB>
+__global__ void __launch_bounds__(256, VB == 4 ? 4 : 3) k_proj_tile(const TIn* __restrict__ C, int64_t m, int64_t n,
+                                                   const float* __restrict__ X, int ldx, int b, TOut* __restrict__ S,
+                                                   int64_t lds) {
+  constexpr int TN = 64, RC = 32, BP = 16 * VB;
+  __shared__ float Cs[RC][TN];
+  __shared__ float Xs[RC][BP];
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int64_t col0 = (int64_t)blockIdx.x * TN;
+  float acc[VB][4] = {};
+  constexpr int NC = RC * TN / 256, NX = RC * BP / 256;   // tile entries per thread
+  for (int64_t i0 = 0; i0 < m; i0 += RC) {
+    uint32_t cl[NC];                                      // every load in flight before the first store
+    float xl[NX];
+#pragma unroll
+    for (int u = 0; u < NC; ++u) {
+      const int e = threadIdx.x + 256 * u, r = e / TN, c = e % TN;
+      cl[u] = (i0 + r < m && col0 + c < n) ? ld_raw(C + (i0 + r) * n + col0 + c) : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < NX; ++u) {
+      const int e = threadIdx.x + 256 * u, r = e / BP, c = e % BP;
+      xl[u] = (i0 + r < m && c < b) ? X[(i0 + r) * ldx + c] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < NC; ++u) {
+      const int e = threadIdx.x + 256 * u;
+      Cs[e / TN][e % TN] = from_raw<TIn>(cl[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < NX; ++u) {
+      const int e = threadIdx.x + 256 * u;
+      Xs[e / BP][e % BP] = xl[u];
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int r = 0; r < RC; ++r) {
+      float cv[4], xv[VB];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) cv[u] = Cs[r][tx + 16 * u];
+#pragma unroll
+      for (int v = 0; v < VB; ++v) xv[v] = Xs[r][ty + 16 * v];
+#pragma unroll
+      for (int v = 0; v < VB; ++v)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[v][u] = fmaf(xv[v], cv[u], acc[v][u]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int v = 0; v < VB; ++v) {
+    const int row = ty + 16 * v;
+    if (row >= b) continue;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t col = col0 + tx + 16 * u;
+      if (col < n) st_elem(S, (int64_t)row * lds + col, acc[v][u]);
+    }
+  }
+}
+
+// Where a CTA of 64 columns is the faster form.  Above 48 columns of X and
+// rows, since four or eight warps would read each element of C for themselves
+// (64 x 262,144 at b = 60: 81 us, 105 by the columns' form).  And for fewer
+// than 128 x 152 columns, which leave the columns' form to a few rows per
+// group and their sums: 20 x 504 at b = 14 2.6 us against 5.2, 130 x 8,069 at
+// b = 30 8.1 against 12.2; the wider groups of 160 rows on, and 21 to 24
+// columns, are as fast there or faster.
+bool proj_tile(int64_t m, int64_t n, int b, int splits) {
+  if (m > 256 || splits != 1) return false;
+  if (b > 48 && m > 48) return true;
+  if (n >= 128 * 152) return false;
+  return m <= 64 || b > 24 || (b > 12 && b <= 20 && m <= 160);
+}
+
+// Row groups of a CTA.  Two CTAs an SM (narrow outputs): as few as give the
+// chip both.  One: the least time by rounds of CTAs x (rows of a group + 40,
+// the start and the sums of a CTA); asking for 304 CTAs of kernels that an SM
+// holds one of left a second round of few (50 x 20,973 at b = 30: 164 CTAs
+// 16.6 us, 82 of them 10.4).
+int proj_row_groups(int64_t n, int64_t rows_per, int splits, int CG, int held) {
+  constexpr int NC = PJ_NC;
+  auto ctas = [&](int rg) { return ceil_div(n, (8 / (CG * rg)) * 32 * NC) * splits; };
+  int RG = 1;
+  if (held == 2) {
+    while (CG * RG < 8 && rows_per >= 16 * RG && ctas(RG) < 2 * 152) RG *= 2;
+    return RG;
+  }
+  int64_t least = -1;
+  for (int rg = 1; CG * rg <= 8 && (rg == 1 || rows_per >= 8 * rg); rg *= 2) {
+    const int64_t t = ceil_div(ctas(rg), 152) * (ceil_div(rows_per, rg) + 40);
+    if (least < 0 || t <= least) {
+      least = t;
+      RG = rg;
+    }
+  }
+  return RG;
+}
+
+template <typename TIn, typename TOut, int TC, bool VEC>
 cudaError_t launch_proj(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b, TOut* S, int64_t lds,
                         int64_t rows_per, int splits, int64_t split_stride, int CG, cudaStream_t st) {
   constexpr int NC = PJ_NC;
-  // narrow outputs: two CTAs an SM; the wide ones hold their 64 or 80 sums and
-  // 64 loads in one
-  constexpr int FR = TC >= 16 ? 8 : 4, CTAS = TC >= 16 ? 1 : 2;
-  // as few row groups as give the chip two CTAs an SM
-  int RG = 1;
-  while (CG * RG < 8 && rows_per >= 16 * RG && ceil_div(n, (8 / (CG * RG)) * 32 * NC) * splits < 2 * 152) RG *= 2;
+  // narrow outputs: two CTAs an SM; the wide ones hold their 48 to 96 sums and
+  // 64 loads in one, as do 12 columns of rows that are read element by element
+  // (with their column offsets they spilled at 128 registers: b = 10, rows not
+  // aligned, BF16 0.77 of the time, 21 to 24 0.73)
+  constexpr bool kOne = TC >= 16 || (TC == 12 && !VEC);
+  constexpr int FR = kOne ? 8 : 4, CTAS = kOne ? 1 : 2;
+  const int RG = proj_row_groups(n, rows_per, splits, CG, CTAS);
   const int cols = (8 / (CG * RG)) * 32 * NC;
-  const bool vec = n % 4 == 0 && lds % 4 == 0 && split_stride % 4 == 0 &&
-                   reinterpret_cast<uintptr_t>(C) % (4 * sizeof(TIn)) == 0 &&
-                   reinterpret_cast<uintptr_t>(S) % (4 * sizeof(TOut)) == 0;
   const bool x16 = b % 4 == 0 && ldx % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0;
   const size_t smem = sizeof(float) * (size_t)imax(RG * 2 * PJ_RK * CG * TC, RG > 1 ? (256 / RG) * NC * TC : 0);
   const dim3 grid((unsigned)ceil_div(n, cols), (unsigned)splits);
-  if (vec)
-    k_proj<TIn, TOut, TC, FR, CTAS, true><<<grid, 256, smem, st>>>(C, m, n, X, ldx, b, S, lds, rows_per, split_stride,
-                                                                  CG, RG, x16);
-  else
-    k_proj<TIn, TOut, TC, FR, CTAS, false><<<grid, 256, smem, st>>>(C, m, n, X, ldx, b, S, lds, rows_per,
-                                                                   split_stride, CG, RG, x16);
+  k_proj<TIn, TOut, TC, FR, CTAS, VEC><<<grid, 256, smem, st>>>(C, m, n, X, ldx, b, S, lds, rows_per, split_stride,
+                                                               CG, RG, x16);
   return cudaGetLastError();
 }
 
 template <typename TIn, typename TOut>
 cudaError_t proj_dispatch(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b, TOut* S, int64_t lds,
                           int64_t rows_per, int splits, int64_t split_stride, cudaStream_t st) {
-#define TTR_PJ(TC, CG) return launch_proj<TIn, TOut, TC>(C, m, n, X, ldx, b, S, lds, rows_per, splits, split_stride, CG, st)
-  if (b <= 4) TTR_PJ(4, 1);
-  if (b <= 8) TTR_PJ(8, 1);
-  if (b <= 12) TTR_PJ(12, 1);
-  if (b <= 16) TTR_PJ(16, 1);
-  if (b <= 20) TTR_PJ(20, 1);
-  if (b <= 24) TTR_PJ(12, 2);
-  if (b <= 32) TTR_PJ(16, 2);
-  if (b <= 40) TTR_PJ(20, 2);
-  if (b <= 48) TTR_PJ(12, 4);
-  if (b <= 64) TTR_PJ(16, 4);
+  if (b > 64) return cudaErrorInvalidValue;
+  if (proj_tile(m, n, b, splits)) {
+    const unsigned ctas = (unsigned)ceil_div(n, 64);
+    if (b <= 16) k_proj_tile<TIn, TOut, 1><<<ctas, 256, 0, st>>>(C, m, n, X, ldx, b, S, lds);
+    else if (b <= 32) k_proj_tile<TIn, TOut, 2><<<ctas, 256, 0, st>>>(C, m, n, X, ldx, b, S, lds);
+    else k_proj_tile<TIn, TOut, 4><<<ctas, 256, 0, st>>>(C, m, n, X, ldx, b, S, lds);
+    return cudaGetLastError();
+  }
+  const bool vec = n % 4 == 0 && lds % 4 == 0 && split_stride % 4 == 0 &&
+                   reinterpret_cast<uintptr_t>(C) % (4 * sizeof(TIn)) == 0 &&
+                   reinterpret_cast<uintptr_t>(S) % (4 * sizeof(TOut)) == 0;
+#define TTR_PJ(TC, CG, VEC) \
+  return launch_proj<TIn, TOut, TC, VEC>(C, m, n, X, ldx, b, S, lds, rows_per, splits, split_stride, CG, st)
+#define TTR_PJ2(TC, CG)              \
+  do {                               \
+    if (vec) TTR_PJ(TC, CG, true);   \
+    TTR_PJ(TC, CG, false);           \
+  } while (0)
+  if (b <= 4) TTR_PJ2(4, 1);
+  if (b <= 8) TTR_PJ2(8, 1);
+  if (b <= 12) TTR_PJ2(12, 1);
+  if (b <= 16) TTR_PJ2(16, 1);
+  if (b <= 20) TTR_PJ2(20, 1);
+  if (b <= 24) TTR_PJ2(12, 2);
+  if (b <= 32) TTR_PJ2(16, 2);
+  if (b <= 40) TTR_PJ2(20, 2);
+  if (b <= 48) {
+    // element by element, reading C by four column groups costs more than 24
+    // columns' sums: 200 x 83,885 at b = 45 (BF16) 158 us by four, so 90
+    if (vec) TTR_PJ(12, 4, true);
+    TTR_PJ(24, 2, false);
+  }
+  TTR_PJ2(16, 4);
+#undef TTR_PJ2
 #undef TTR_PJ
-  return cudaErrorInvalidValue;
 }
 
 }  // namespace

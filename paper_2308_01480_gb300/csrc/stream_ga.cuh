@@ -3,22 +3,27 @@
 //
 // Each column tile of C is read from memory once, into shared memory, and
 // used by both products:
-//   1  T = C_tile^T X: a lane owns two columns, a warp TC1 columns of X (one
-//      of CG1 groups) and every RS-th row; the RS partial tiles are added in
-//      order.  X is read as broadcasts.
+//   1  T = C_tile^T X: a lane owns two columns (one of a 32-column tile), a
+//      warp TC1 columns of X (one of CG1 groups) and every RS-th row; the RS
+//      partial tiles are added in order.  X is read as broadcasts.
 //   2  Z += C_tile T^T as rows times rows (simt_tile.cuh): TR x TC register
 //      tiles fed by 16-byte loads along the tile's columns, RT row tiles x
 //      CT column tiles x KG groups of columns, kept in registers over all of
 //      the CTA's tiles; the group sums are added in order at the end.
 // Both phases do four or more multiply-adds per shared-memory instruction;
 // the tile's width (128 columns, 64 above 128 rows) leaves room for two or
-// more CTAs an SM, so that one CTA's loads overlap another's products.
+// more CTAs an SM, so that one CTA's loads overlap another's products.  A tile
+// is a long chain for one CTA: unfoldings of up to 2,048 columns take tiles of
+// 32 (120 x 504 at b = 45 24.4 -> 14.7), and above 128 rows and 12 columns of
+// X also where 64 leave SMs without one (n < 9,728; 256 x 4,096 at b = 32
+// 31.9 -> 18.9).  Wider tiles have fewer partials to add.
 // Before, both products loaded their operands as scalars (one per 1 to 2
 // multiply-adds for narrow blocks).  Measured (FP32, us): 45 x 4,100,625 at
 // b = 6 1,230 -> 287 (738 MB, 2.6 TB/s; BF16, rows not aligned, 1,178 ->
 // 287), 180 x 91,125 at b = 6 101 -> 31, 256 x 32,768 at b = 13 54 -> 34.
 #pragma once
 
+#include "cluster_la.cuh"
 #include "common.cuh"
 #include "kernels.h"
 #include "simt_tile.cuh"
@@ -34,14 +39,16 @@ struct GaShape {
   int cw, rs;       // phase 1: warps across the tile's columns, row splits
   int kg;           // phase 2: groups over the tile's columns
   int mp, bp1, bn, ld;
+  int ls;           // row stride of the group sums
   size_t off_x, off_t, off_p, smem;   // floats, floats, floats, bytes
 };
 
-inline bool ga_shape(int64_t m, int b, GaShape* s) {
+inline bool ga_shape(int64_t m, int64_t n, int b, GaShape* s) {
   if (m < 1 || m > 256 || b < 1 || b > 48) return false;
   s->rt = m <= 64 ? 8 : m <= 128 ? 16 : 32;
-  s->tr = m <= 32 ? 4 : m <= 48 ? 6 : 8;
-  s->tn = m <= 128 ? 128 : 64;
+  const bool tiny = n <= 2048;
+  s->tr = tiny ? 8 : m <= 32 ? 4 : m <= 48 ? 6 : 8;
+  s->tn = tiny ? 32 : m <= 128 ? 128 : b <= 12 || ceil_div(n, 64) >= 152 ? 64 : 32;
   if (b <= 4) { s->tc = 4; s->ct = 1; s->tc1 = 4; s->cg1 = 1; }
   else if (b <= 6) { s->tc = 6; s->ct = 1; s->tc1 = 8; s->cg1 = 1; }
   else if (b <= 8) { s->tc = 8; s->ct = 1; s->tc1 = 8; s->cg1 = 1; }
@@ -50,9 +57,9 @@ inline bool ga_shape(int64_t m, int b, GaShape* s) {
   else if (b <= 24) { s->tc = 6; s->ct = 4; s->tc1 = 12; s->cg1 = 2; }
   else if (b <= 32) { s->tc = 8; s->ct = 4; s->tc1 = 8; s->cg1 = 4; }
   else { s->tc = 6; s->ct = 8; s->tc1 = 12; s->cg1 = 4; }
-  s->cw = s->tn / 64;
+  s->cw = s->tn >= 64 ? s->tn / 64 : 1;
   s->rs = 8 / (s->cw * s->cg1);
-  s->kg = 256 / (s->rt * s->ct);
+  s->kg = (int)imin(256 / (s->rt * s->ct), s->tn / 4);
   s->mp = s->rt * s->tr;
   s->bp1 = s->tc1 * s->cg1;
   s->bn = s->tc * s->ct;
@@ -61,7 +68,11 @@ inline bool ga_shape(int64_t m, int b, GaShape* s) {
   s->off_t = s->off_x + (size_t)((m + 3) / 4 * 4) * s->bp1;
   s->off_p = s->off_t + (size_t)s->bn * s->ld;
   const size_t tiles = s->off_p + (s->rs > 1 ? (size_t)s->rs * s->bp1 * s->tn : 0);
-  const size_t sums = (size_t)256 * s->tr * s->tc;
+  // lanes hold consecutive rows: an odd stride keeps their stores in different
+  // banks (a stride of bn = 32 made them take turns: 256 x 4,096 at b = 32
+  // 35 us, so 28 with tiles of 64)
+  s->ls = s->bn | 1;
+  const size_t sums = (size_t)s->kg * s->mp * s->ls;
   s->smem = sizeof(float) * (tiles > sums ? tiles : sums);
   return true;
 }
@@ -120,8 +131,21 @@ struct GaLoad {
   }
 };
 
+// The m x wv column tile of an FP32 C with aligned rows straight to shared
+// memory, every copy in flight (columns past wv become zero).  Element by
+// element (rows not aligned) this was slower than loads in parts.
+template <int TN>
+__device__ __forceinline__ void ga_copy_async(float* Cs, const float* __restrict__ C, int64_t n, int m, int wv) {
+  constexpr int LD = TN + 4, PER = TN / 4;
+  const int c = (threadIdx.x % PER) * 4;
+  const bool in = c < wv;                   // all four or none: n is a multiple of four
+  for (int row = threadIdx.x / PER; row < m; row += 256 / PER)
+    cp_async16z(Cs + row * LD + c, in ? C + (int64_t)row * n + c : C, in);
+}
+
 // PF > 0: the whole next tile (PF elements a thread) is loaded into registers
-// while the current one is multiplied; 0: loaded in parts of 8 elements.
+// while the current one is multiplied; 0: copied asynchronously (FP32, rows
+// aligned) or loaded in parts of 16 elements.
 template <typename TIn, int TR, int TC, int TC1, int TN, int PF>
 __global__ void __launch_bounds__(256, 2) k_ga(const TIn* __restrict__ C, int64_t m64, int64_t n,
                                                const float* __restrict__ X, int ldx, int b, float* __restrict__ P,
@@ -134,9 +158,20 @@ __global__ void __launch_bounds__(256, 2) k_ga(const TIn* __restrict__ C, int64_
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   constexpr int LD = TN + 4;
   const int m = (int)m64, BP1 = p.bp1;
-  for (int e = tid; e < m * BP1; e += 256) {
-    const int r = e / BP1, c = e - r * BP1;
-    Xs[e] = c < b ? X[(int64_t)r * ldx + c] : 0.f;
+  // X, all copies in flight beside the first tile's
+  {
+    const int dr = 256 / BP1, dc = 256 - dr * BP1;
+    int r = tid / BP1, c = tid - r * BP1;
+    for (int e = tid; e < m * BP1; e += 256) {
+      const bool in = c < b;
+      cp_async4(Xs + e, in ? X + (int64_t)r * ldx + c : X, in);
+      r += dr;
+      c += dc;
+      if (c >= BP1) {
+        c -= BP1;
+        ++r;
+      }
+    }
   }
   for (int e = tid; e < (p.mp - m) * LD; e += 256) Cs[m * LD + e] = 0.f;
   for (int e = tid; e < p.bn * LD; e += 256) Ts[e] = 0.f;
@@ -152,7 +187,7 @@ __global__ void __launch_bounds__(256, 2) k_ga(const TIn* __restrict__ C, int64_
   const int64_t ntiles = ceil_div(n, TN);
   const int64_t t_beg = (int64_t)blockIdx.x * tiles_per_cta, t_end = imin(ntiles, t_beg + tiles_per_cta);
   const int ks = TN / (4 * p.kg);
-  GaLoad<TIn, TN, PF ? PF : 8> ld;
+  GaLoad<TIn, TN, PF ? PF : 16> ld;
   if constexpr (PF > 0) {
     if (t_beg < t_end) ld.load(C + t_beg * TN, n, m, (int)imin(TN, n - t_beg * TN), vec);
   }
@@ -162,18 +197,22 @@ __global__ void __launch_bounds__(256, 2) k_ga(const TIn* __restrict__ C, int64_
     __syncthreads();
     if constexpr (PF > 0) {
       ld.store(Cs, m, vec);
+    } else if (sizeof(TIn) == 4 && vec) {
+      ga_copy_async<TN>(Cs, reinterpret_cast<const float*>(C) + c0, n, m, wv);
     } else {
-      GaLoad<TIn, TN, 8> part;
-      for (int r0 = 0; r0 < m; r0 += GaLoad<TIn, TN, 8>::rows) {
+      GaLoad<TIn, TN, 16> part;
+      for (int r0 = 0; r0 < m; r0 += GaLoad<TIn, TN, 16>::rows) {
         part.load(C + (int64_t)r0 * n + c0, n, m - r0, wv, vec);
         part.store(Cs + r0 * LD, m - r0, vec);
       }
     }
+    cp_async_wait_all();                    // the tile's copies, and X's before the first
     __syncthreads();
     if constexpr (PF > 0) {
       if (tile + 1 < t_end) ld.load(C + c0 + TN, n, m, (int)imin(TN, n - c0 - TN), vec);
     }
     {
+      constexpr bool kTwo = TN >= 64;          // columns of a lane
       float t0[TC1], t1[TC1];
 #pragma unroll
       for (int c = 0; c < TC1; ++c) t0[c] = t1[c] = 0.f;
@@ -182,7 +221,7 @@ __global__ void __launch_bounds__(256, 2) k_ga(const TIn* __restrict__ C, int64_
       const int cstep = p.rs * LD, xstep = p.rs * BP1;
 #pragma unroll 4
       for (int i = rs0; i < m; i += p.rs, cc += cstep, xx += xstep) {
-        const float a0 = cc[0], a1 = cc[32];
+        const float a0 = cc[0], a1 = kTwo ? cc[32] : 0.f;
 #pragma unroll
         for (int c4 = 0; c4 < TC1 / 4; ++c4) {
           const float4 x = *reinterpret_cast<const float4*>(xx + 4 * c4);
@@ -190,10 +229,12 @@ __global__ void __launch_bounds__(256, 2) k_ga(const TIn* __restrict__ C, int64_
           t0[4 * c4 + 1] = fmaf(a0, x.y, t0[4 * c4 + 1]);
           t0[4 * c4 + 2] = fmaf(a0, x.z, t0[4 * c4 + 2]);
           t0[4 * c4 + 3] = fmaf(a0, x.w, t0[4 * c4 + 3]);
-          t1[4 * c4] = fmaf(a1, x.x, t1[4 * c4]);
-          t1[4 * c4 + 1] = fmaf(a1, x.y, t1[4 * c4 + 1]);
-          t1[4 * c4 + 2] = fmaf(a1, x.z, t1[4 * c4 + 2]);
-          t1[4 * c4 + 3] = fmaf(a1, x.w, t1[4 * c4 + 3]);
+          if constexpr (kTwo) {
+            t1[4 * c4] = fmaf(a1, x.x, t1[4 * c4]);
+            t1[4 * c4 + 1] = fmaf(a1, x.y, t1[4 * c4 + 1]);
+            t1[4 * c4 + 2] = fmaf(a1, x.z, t1[4 * c4 + 2]);
+            t1[4 * c4 + 3] = fmaf(a1, x.w, t1[4 * c4 + 3]);
+          }
         }
       }
       if (p.rs > 1) {
@@ -201,7 +242,7 @@ __global__ void __launch_bounds__(256, 2) k_ga(const TIn* __restrict__ C, int64_
 #pragma unroll
         for (int c = 0; c < TC1; ++c) {
           tp[(cg * TC1 + c) * TN] = t0[c];
-          tp[(cg * TC1 + c) * TN + 32] = t1[c];
+          if constexpr (kTwo) tp[(cg * TC1 + c) * TN + 32] = t1[c];
         }
         __syncthreads();
         for (int e = tid; e < b * TN; e += 256) {
@@ -215,29 +256,33 @@ __global__ void __launch_bounds__(256, 2) k_ga(const TIn* __restrict__ C, int64_
         for (int c = 0; c < TC1; ++c)
           if (cg * TC1 + c < b) {
             Ts[(cg * TC1 + c) * LD + cw * 64 + lane] = t0[c];
-            Ts[(cg * TC1 + c) * LD + cw * 64 + lane + 32] = t1[c];
+            if constexpr (kTwo) Ts[(cg * TC1 + c) * LD + cw * 64 + lane + 32] = t1[c];
           }
       }
     }
     __syncthreads();
-    for (int s = 0; s < ks; ++s) {
-      const int k4 = 4 * (kg + s * p.kg);
-      simt::nt_step<TR, TC>(acc, Cs + rt * LD + k4, p.rt * LD, Ts + ct * LD + k4, p.ct * LD);
+    if (kg < p.kg) {                        // a short tile has fewer groups than the CTA
+      for (int s = 0; s < ks; ++s) {
+        const int k4 = 4 * (kg + s * p.kg);
+        simt::nt_step<TR, TC>(acc, Cs + rt * LD + k4, p.rt * LD, Ts + ct * LD + k4, p.ct * LD);
+      }
     }
   }
   // group sums in group order
   __syncthreads();
+  if (kg < p.kg) {
 #pragma unroll
-  for (int u = 0; u < TR; ++u)
+    for (int u = 0; u < TR; ++u)
 #pragma unroll
-    for (int v = 0; v < TC; ++v)
-      ga_sm[((size_t)kg * p.mp + rt + p.rt * u) * p.bn + ct + p.ct * v] = acc[u][v];
+      for (int v = 0; v < TC; ++v)
+        ga_sm[((size_t)kg * p.mp + rt + p.rt * u) * p.ls + ct + p.ct * v] = acc[u][v];
+  }
   __syncthreads();
   float* out = P + (int64_t)blockIdx.x * m * b;
   for (int e = tid; e < m * b; e += 256) {
     const int i = e / b, c = e - i * b;
     float s = 0.f;
-    for (int g = 0; g < p.kg; ++g) s += ga_sm[((size_t)g * p.mp + i) * p.bn + c];
+    for (int g = 0; g < p.kg; ++g) s += ga_sm[((size_t)g * p.mp + i) * p.ls + c];
     out[e] = s;
   }
 }
@@ -279,14 +324,15 @@ template <typename TIn>
 cudaError_t simt_ga_with_ctas(const TIn* C, int64_t m, int64_t n, const float* X, int ldx, int b,
                               float* partials, int64_t max_ctas, float* out, int64_t ldo, cudaStream_t st) {
   GaShape s;
-  if (max_ctas < 1 || !ga_shape(m, b, &s)) return cudaErrorInvalidValue;
+  if (max_ctas < 1 || !ga_shape(m, n, b, &s)) return cudaErrorInvalidValue;
   int64_t tpc;
   int ctas;
   ga_plan(s, n, max_ctas, &tpc, &ctas);
   {
     ProfScope prof("gram_apply_simt", st, (double)m * n * sizeof(TIn) + (double)m * b * 4, 4.0 * m * n * b);
     note_launch("gram_apply_simt");
-    const cudaError_t e = s.tr == 4     ? ga_dispatch<TIn, 4, 128, 16>(C, m, n, X, ldx, b, partials, tpc, ctas, s, st)
+    const cudaError_t e = s.tn == 32    ? ga_dispatch<TIn, 8, 32, 0>(C, m, n, X, ldx, b, partials, tpc, ctas, s, st)
+                          : s.tr == 4   ? ga_dispatch<TIn, 4, 128, 16>(C, m, n, X, ldx, b, partials, tpc, ctas, s, st)
                           : s.tr == 6   ? ga_dispatch<TIn, 6, 128, 24>(C, m, n, X, ldx, b, partials, tpc, ctas, s, st)
                           : s.rt == 8   ? ga_dispatch<TIn, 8, 128, 32>(C, m, n, X, ldx, b, partials, tpc, ctas, s, st)
                           : s.tn == 128 ? ga_dispatch<TIn, 8, 128, 0>(C, m, n, X, ldx, b, partials, tpc, ctas, s, st)

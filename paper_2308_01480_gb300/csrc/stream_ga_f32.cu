@@ -8,7 +8,7 @@ bool simt_ga_fused_ok(int64_t m, int b) { return m <= 256 && b <= 48 && ceil_div
 
 int64_t simt_ga_partials(int64_t m, int64_t n, int b) {
   GaShape s;
-  if (!ga_shape(m, b, &s)) return 0;
+  if (!ga_shape(m, n, b, &s)) return 0;
   int64_t tpc;
   int ctas;
   ga_plan(s, n, int64_t(1) << 30, &tpc, &ctas);

@@ -356,7 +356,7 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
     double* Hd = (double*)(ws + P.off_Hd);
     double* dfp = (double*)(ws + P.off_dfp);
     TTR_CUDA(ttr::gram_df<TIn>(C, (int)M.m, M.n, M.n, dfp, Hd, st));
-    TTR_CUDA(ttr::launch_rr_svd(Hd, (int)M.m, r, nullptr, M.m, 0, U, nullptr, status, st));
+    TTR_CUDA(ttr::launch_rr_svd(Hd, (int)M.m, r, nullptr, M.m, 0, U, status, st));
   } else if (M.gram_route) {
     float* G = (float*)(ws + P.off_G);
     if (use_tc && M.m <= 128)
@@ -368,9 +368,9 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
       if (rs != TT_OK) return rs;
     }
     if (ttr::eig_top_ok((int)M.m))
-      TTR_CUDA(ttr::launch_rr_fast(nullptr, G, M.m, M.m, (int)M.m, r, 1, small, U, nullptr, st));
+      TTR_CUDA(ttr::launch_rr_fast(nullptr, G, M.m, M.m, (int)M.m, r, 1, small, U, st));
     else
-      TTR_CUDA(ttr::launch_rayleigh_ritz(nullptr, G, M.m, M.m, (int)M.m, r, 1, small, U, nullptr, st));
+      TTR_CUDA(ttr::launch_rayleigh_ritz(nullptr, G, M.m, M.m, (int)M.m, r, 1, small, U, st));
   } else if (M.gram_cols) {
     // exhaustion with D = n < m: the Krylov basis would span range(C), so
     // Rayleigh-Ritz would return the exact top-r left singular vectors;
@@ -577,11 +577,11 @@ tt_status run_mode(const Plan& P, int k, const TIn* C, char* ws, int* status, co
         TTR_CUDA((ttr::simt_proj<TIn, float>(C, M.m, M.n, Q + c0, kq, cw, Bm + (size_t)c0 * M.n, M.n, st, nullptr)));
       }
       TTR_CUDA(ttr::gram_df<float>(Bm, kq, M.n, M.n, dfp, Hd, st));
-      TTR_CUDA(ttr::launch_rr_svd(Hd, kq, r, Q, M.m, kq, U, nullptr, status, st));
+      TTR_CUDA(ttr::launch_rr_svd(Hd, kq, r, Q, M.m, kq, U, status, st));
     } else if (ttr::eig_top_ok(kq)) {
-      TTR_CUDA(ttr::launch_rr_fast(Q, W, kq, M.m, kq, r, 0, small, U, nullptr, st));
+      TTR_CUDA(ttr::launch_rr_fast(Q, W, kq, M.m, kq, r, 0, small, U, st));
     } else {
-      TTR_CUDA(ttr::launch_rayleigh_ritz(Q, W, kq, M.m, kq, r, 0, small, U, nullptr, st));
+      TTR_CUDA(ttr::launch_rayleigh_ritz(Q, W, kq, M.m, kq, r, 0, small, U, st));
     }
     }
   }

@@ -489,14 +489,14 @@ __global__ void __launch_bounds__(EIG_THREADS) k_eig_top(const float* __restrict
     for (int j = threadIdx.x; j < r; j += blockDim.x) evals[j] = S.lam[j];
 }
 
-// U (m x r) = Q (m x k, ld ldq) V (k x r); also written to core (same layout).
+// U (m x r) = Q (m x k, ld ldq) V (k x r).
 // V and the CTA's rows of Q are staged in shared memory with sixteen loads
 // of each thread in flight at a time; each U entry is then one FMA chain over
 // t = 0..k-1.
 template <typename TQ>
 __global__ void __launch_bounds__(256) k_apply_basis(const TQ* __restrict__ Q, int64_t ldq, int64_t m, int k,
                                                      const float* __restrict__ V, int r, float* __restrict__ U,
-                                                     float* __restrict__ core, int64_t rows_per_cta) {
+                                                     int64_t rows_per_cta) {
   constexpr int NT = 256, NL = 16;
   extern __shared__ float sm[];
   float* Vs = sm;                     // [k][r]
@@ -531,7 +531,6 @@ __global__ void __launch_bounds__(256) k_apply_basis(const TQ* __restrict__ Q, i
     float s = 0.f;
     for (int t = 0; t < k; ++t) s = fmaf(qi[t], Vs[t * r + j], s);
     U[i * r + j] = s;
-    if (core) core[i * r + j] = s;
   }
 }
 
@@ -598,20 +597,20 @@ static cudaError_t launch_tn(const TA* A, int64_t lda, int ka, const TB* B, int6
 
 template <typename TQ>
 static cudaError_t apply_basis_t(const TQ* Q, int64_t ldq, int64_t m, int k, const float* V, int r, float* U,
-                                 float* core, cudaStream_t st) {
+                                 cudaStream_t st) {
   int64_t rpc = 8;
   const int ctas = (int)ceil_div(m, rpc);
   const size_t smem = sizeof(float) * ((size_t)k * r + (size_t)rpc * k);
   raise_smem_limit(k_apply_basis<TQ>);
   ProfScope prof("apply_basis", st, 0, 2.0 * m * k * r);
   note_launch("apply_basis");
-  k_apply_basis<TQ><<<ctas, 256, smem, st>>>(Q, ldq, m, k, V, r, U, core, rpc);
+  k_apply_basis<TQ><<<ctas, 256, smem, st>>>(Q, ldq, m, k, V, r, U, rpc);
   return cudaGetLastError();
 }
 
 cudaError_t launch_apply_basis(const float* Q, int64_t ldq, int64_t m, int k, const float* V, int r, float* U,
-                               float* core, cudaStream_t st) {
-  return apply_basis_t(Q, ldq, m, k, V, r, U, core, st);
+                               cudaStream_t st) {
+  return apply_basis_t(Q, ldq, m, k, V, r, U, st);
 }
 
 // Rayleigh-Ritz: H = Q^T W (or H = G when Q is the identity), top-r
@@ -621,7 +620,7 @@ size_t rr_fast_scratch_floats(int64_t m, int k, int r) {
 }
 
 cudaError_t launch_rr_fast(const float* Q, const float* W, int64_t ld, int64_t m, int k, int r, int identity_q,
-                           float* scratch, float* U, float* core, cudaStream_t st) {
+                           float* scratch, float* U, cudaStream_t st) {
   float* parts = scratch;
   float* H = parts + tn_parts_floats(m, k, k);
   float* V = H + (size_t)k * k;
@@ -641,12 +640,8 @@ cudaError_t launch_rr_fast(const float* Q, const float* W, int64_t ld, int64_t m
   // Q = I (m == k): U = V
   e = launch_eig_top(Hsrc, ldh, k, r, identity_q ? U : V, es, nullptr, st);
   if (e != cudaSuccess) return e;
-  if (identity_q) {
-    if (core)
-      e = cudaMemcpyAsync(core, U, sizeof(float) * (size_t)m * r, cudaMemcpyDeviceToDevice, st);
-    return e;
-  }
-  return launch_apply_basis(Q, ld, m, k, V, r, U, core, st);
+  if (identity_q) return e;
+  return launch_apply_basis(Q, ld, m, k, V, r, U, st);
 }
 
 // Exhaustion with D = n < m (the Krylov basis would span range(C)): the
@@ -667,7 +662,7 @@ cudaError_t launch_colgram(const T* C, int64_t m, int n, int r, float* scratch, 
   if (e != cudaSuccess) return e;
   e = launch_eig_top(G, n, n, r, V, es, nullptr, st);
   if (e != cudaSuccess) return e;
-  return apply_basis_t(C, n, m, n, V, r, Y, nullptr, st);
+  return apply_basis_t(C, n, m, n, V, r, Y, st);
 }
 
 template cudaError_t launch_colgram<float>(const float*, int64_t, int, int, float*, float*, cudaStream_t);

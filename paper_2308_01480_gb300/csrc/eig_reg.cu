@@ -62,12 +62,6 @@ __device__ __forceinline__ float warp_max_f(float v) {
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
-__device__ __forceinline__ int warp_min_i(int v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
 // Pivoted LU of T - lam I, one thread per vector: row i of w holds
 // (1 / pivot, two upper diagonals, multiplier), bit i & 7 of ex[i / 8] whether
 // rows were exchanged; tiny pivots replaced by +-tiny.  Rows k .. kp - 1 (kp a

@@ -157,14 +157,14 @@ template <typename T>
 cudaError_t gram_df(const T* B, int k, int64_t n, int64_t ldb, double* partials, double* H, cudaStream_t st);
 bool rr_svd_ok(int k, int r);
 cudaError_t launch_rr_svd(const double* H, int k, int r, const float* Q, int64_t m, int64_t ldq, float* U,
-                          float* core, int* status, cudaStream_t st);
+                          int* status, cudaStream_t st);
 bool eig_top_ok(int k);
 size_t rr_fast_scratch_floats(int64_t m, int k, int r);
 size_t eig_scratch_floats(int k, int r);
 cudaError_t launch_eig_top(const float* H, int64_t ldh, int k, int r, float* V, float* scratch, float* evals,
                            cudaStream_t st);
 cudaError_t launch_rr_fast(const float* Q, const float* W, int64_t ld, int64_t m, int k, int r, int identity_q,
-                           float* scratch, float* U, float* core, cudaStream_t st);
+                           float* scratch, float* U, cudaStream_t st);
 size_t rr_scratch_floats(int k);
 // exhaustion with D = n < m: Y = C V' (m x r), V' the top-r eigenvectors of
 // C^T C (n x n, n <= 224); scratch: colgram_scratch_floats(m, n, r)
@@ -172,7 +172,7 @@ size_t colgram_scratch_floats(int64_t m, int n, int r);
 template <typename T>
 cudaError_t launch_colgram(const T* C, int64_t m, int n, int r, float* scratch, float* Y, cudaStream_t st);
 cudaError_t launch_rayleigh_ritz(const float* Q, const float* W, int64_t ld, int64_t m, int k, int r,
-                                 int identity_q, float* scratch, float* U, float* core, cudaStream_t st);
+                                 int identity_q, float* scratch, float* U, cudaStream_t st);
 // The last core (the last remainder of dtype TT_F32/TT_BF16, last_count
 // entries) and a non-finite check of it and of cores[0..ncores) (counts[k]
 // entries each), one launch; ncores <= kFinaliseMaxCores.

@@ -265,8 +265,7 @@ __global__ void __launch_bounds__(256) k_permute_rows(const TS* __restrict__ src
 }
 
 struct PermTile {
-  int s;                  // destination mode with the smallest source stride
-  uint32_t S, J;          // sizes of mode s and of the innermost mode
+  uint32_t S, J;          // sizes of mode s (smallest source stride) and of the innermost mode
   uint32_t nts, ntj;      // tiles along each
   FastDiv fts, ftj;
   PermArgs o;             // the other modes, in destination order
@@ -386,7 +385,6 @@ static cudaError_t permute_typed(const TS* src, TD* dst, int64_t total, PermArgs
     return cudaGetLastError();
   }
   PermTile p = {};
-  p.s = s;
   p.S = (uint32_t)c.ddims[s];
   p.J = (uint32_t)c.ddims[last];
   p.ss = c.sstride[s];

@@ -160,7 +160,7 @@ __host__ __device__ inline size_t rs_smem_bytes(int k) {
 
 __global__ void __launch_bounds__(RS_THREADS, 1)
 k_rr_svd(const double* __restrict__ Hg, int k, int r, const float* __restrict__ Q, int64_t m, int64_t ldq,
-         float* __restrict__ U, float* __restrict__ core, int* status) {
+         float* __restrict__ U, int* status) {
   extern __shared__ __align__(16) unsigned char smraw[];
   double* Lp = reinterpret_cast<double*>(smraw);                      // packed lower, row i at i (i + 1) / 2
   const int ldw = k | 1;
@@ -409,7 +409,6 @@ k_rr_svd(const double* __restrict__ Hg, int k, int r, const float* __restrict__ 
       s = y[iperm[i]];
     }
     U[x] = s;
-    if (core) core[x] = s;
   }
   (void)status;
 }
@@ -449,14 +448,14 @@ bool rr_svd_ok(int k, int r) {
 }
 
 cudaError_t launch_rr_svd(const double* H, int k, int r, const float* Q, int64_t m, int64_t ldq, float* U,
-                          float* core, int* status, cudaStream_t st) {
+                          int* status, cudaStream_t st) {
   if (!rr_svd_ok(k, r)) return cudaErrorInvalidValue;
   const size_t smem = rs_smem_bytes(k);
   cudaError_t e = raise_smem_limit(k_rr_svd);
   if (e != cudaSuccess) return e;
   ProfScope prof("rr_svd", st, 0, 0);
   note_launch("rr_svd");
-  k_rr_svd<<<1, RS_THREADS, smem, st>>>(H, k, r, Q, m, ldq, U, core, status);
+  k_rr_svd<<<1, RS_THREADS, smem, st>>>(H, k, r, Q, m, ldq, U, status);
   return cudaGetLastError();
 }
 

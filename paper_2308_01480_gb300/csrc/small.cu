@@ -267,11 +267,11 @@ k_orth_block(const float* __restrict__ Z, int64_t ldz, int64_t m, int zc, float*
 
 // ------------------------------------------------------------ rayleigh-ritz
 // H = Q^T W (k x k, symmetrised), eigen-decomposed; U = Q V[:, top r]
-// written to U (m x r, row stride r) and to the core (same layout, FP32).
+// written to U (m x r, row stride r).
 // With identity_q, H = W (the Gram C C^T of the exhaustion route) and U = V.
 __global__ void __launch_bounds__(SMALL_THREADS)
 k_rayleigh_ritz(const float* __restrict__ Q, const float* __restrict__ W, int64_t ld, int64_t m, int k,
-                int r, int identity_q, float* Hg, float* Vg, int use_global, float* U, float* core) {
+                int r, int identity_q, float* Hg, float* Vg, int use_global, float* U) {
   extern __shared__ float sm[];
   float* red = sm;               // [64]
   float* cs = red + 64;          // [4 * 128]
@@ -318,7 +318,6 @@ k_rayleigh_ritz(const float* __restrict__ Q, const float* __restrict__ W, int64_
       for (int t = 0; t < k; ++t) s = fmaf(Q[i * ld + t], V[t * ldh + col], s);
     }
     U[e] = s;
-    if (core) core[e] = s;
   }
 }
 
@@ -375,7 +374,7 @@ cudaError_t launch_orth_block(const float* Z, int64_t ldz, int64_t m, int zc, fl
 size_t rr_scratch_floats(int k) { return (size_t)2 * k * (k + 1); }
 
 cudaError_t launch_rayleigh_ritz(const float* Q, const float* W, int64_t ld, int64_t m, int k, int r,
-                                 int identity_q, float* scratch, float* U, float* core, cudaStream_t st) {
+                                 int identity_q, float* scratch, float* U, cudaStream_t st) {
   size_t base = sizeof(float) * (64 + 4 * 128) + sizeof(int) * ((k + 3) & ~3);
   size_t mats = sizeof(float) * 2 * (size_t)k * (k + 1);
   int use_global = (base + mats > 220 * 1024) ? 1 : 0;
@@ -385,7 +384,7 @@ cudaError_t launch_rayleigh_ritz(const float* Q, const float* W, int64_t ld, int
   ProfScope prof("rayleigh_ritz", st, 0, 0);
   note_launch("rayleigh_ritz");
   k_rayleigh_ritz<<<1, SMALL_THREADS, smem, st>>>(Q, W, ld, m, k, r, identity_q, scratch,
-                                                  scratch + (size_t)k * (k + 1), use_global, U, core);
+                                                  scratch + (size_t)k * (k + 1), use_global, U);
   return cudaGetLastError();
 }
 

@@ -79,7 +79,7 @@ __device__ inline void chol_inv_cta(float* G, int ldg, int b, const float* diag0
 // is replaced by 1.
 //
 // The step's latency decides the time, and one warp doing both sweeps in
-// turn pays it twice: b = 30 took 15.1K cycles on one warp, 7.7K on two
+// turn pays it twice: b = 30 alone took 15.1K cycles on one warp, 7.7K on two
 // (bit-identical).
 template <int W>
 struct CholShared {

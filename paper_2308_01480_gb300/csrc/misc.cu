@@ -169,7 +169,9 @@ cudaError_t launch_omega_transpose_any(const float* src, int64_t n, int b, void*
 constexpr int kPermMax = 8;
 constexpr int64_t kPermTileMin = 8;
 
-// n / d for n < 2^31 as a multiply-high, an add and a shift (d >= 1).
+// n / d for n < 2^31 as a multiply-high, an add and a shift (d >= 1), after
+// Granlund and Montgomery, Division by Invariant Integers using Multiplication
+// (1994).
 struct FastDiv {
   uint32_t d, mul, sh;
 };
@@ -279,8 +281,9 @@ struct PermTile {
 // TJ x TSZ tiles: 256 threads read rows of TSZ source-contiguous entries
 // (lane = mode s) into shared memory and write rows of TJ entries (lane = the
 // innermost mode), two to a 4-byte store for BF16 where rows are even (PAIR).
-// The odd row stride keeps both directions free of bank conflicts; 8 to 16
-// loads a thread are in flight.
+// The odd row stride keeps both directions free of bank conflicts, but for the
+// paired stores of 64-entry rows, whose two reads each take two turns (entries
+// 32 apart share a bank); 8 to 16 loads a thread are in flight.
 template <typename TS, typename TD, int TSZ, int TJ, bool PAIR>
 __global__ void __launch_bounds__(256) k_permute_tiles(const TS* __restrict__ src, TD* __restrict__ dst,
                                                        const __grid_constant__ PermTile p) {

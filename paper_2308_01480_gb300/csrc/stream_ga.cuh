@@ -20,7 +20,7 @@
 // Before, both products loaded their operands as scalars (one per 1 to 2
 // multiply-adds for narrow blocks).  Measured (FP32, us): 45 x 4,100,625 at
 // b = 6 1,230 -> 287 (738 MB, 2.6 TB/s; BF16, rows not aligned, 1,178 ->
-// 287), 180 x 91,125 at b = 6 101 -> 31, 256 x 32,768 at b = 13 54 -> 34.
+// 287), 180 x 91,125 at b = 6 101 -> 31, 256 x 32,768 at b = 13 54 -> 29.
 #pragma once
 
 #include "cluster_la.cuh"

@@ -19,8 +19,8 @@
 // (k_proj_tile).
 // Measured (FP32, us; before: 16 x 16 threads with both operands staged in
 // shared memory and no split over rows unless n <= 512): 7680 x 2048 at
-// b = 20 404 -> 31, 800 x 64,000 at b = 20 190 -> 106, 45 x 4,100,625 at
-// b = 6 640 -> 208 (3.5 TB/s); BF16 715 -> 201.  What bounds it now is
+// b = 20 404 -> 25, 800 x 64,000 at b = 20 190 -> 87, 45 x 4,100,625 at
+// b = 6 640 -> 208 (3.5 TB/s); BF16 715 -> 200.  What bounds it now is
 // latency at one to two CTAs an SM.
 #include "cluster_la.cuh"
 #include "common.cuh"
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(256, VB == 4 ? 4 : 3) k_proj_tile(const TIn* _
 
 // Where a CTA of 64 columns is the faster form.  Above 48 columns of X and
 // rows, since four or eight warps would read each element of C for themselves
-// (64 x 262,144 at b = 60: 81 us, 105 by the columns' form).  And for fewer
+// (64 x 262,144 at b = 60: 84 us, 105 by the columns' form).  And for fewer
 // than 128 x 152 columns, which leave the columns' form to a few rows per
 // group and their sums: 20 x 504 at b = 14 2.6 us against 5.2, 130 x 8,069 at
 // b = 30 8.1 against 12.2; the wider groups of 160 rows on, and 21 to 24
@@ -368,7 +368,7 @@ cudaError_t proj_dispatch(const TIn* C, int64_t m, int64_t n, const float* X, in
   if (b <= 40) TTR_PJ2(20, 2);
   if (b <= 48) {
     // element by element, reading C by four column groups costs more than 24
-    // columns' sums: 200 x 83,885 at b = 45 (BF16) 158 us by four, so 90
+    // columns' sums: 200 x 83,885 at b = 45 (BF16) 158 us by four, so 78
     if (vec) TTR_PJ(12, 4, true);
     TTR_PJ(24, 2, false);
   }
